@@ -305,11 +305,11 @@ pm_status pm_get_timings(pm_ctx *ctx, double *ms, int n, int64_t *launches);
  * Errors: INVALID_ARG (force_* outside -2..2), STATE, CUDA. */
 pm_status pm_fft_shapes(pm_ctx *ctx, int32_t force_y, int32_t force_z, int32_t *y_shape, int32_t *z_shape);
 
-/* Shape of the projection's shared-memory bins (Sec. 2.1, the particle-mesh
- * projection): the number of particle records one 8^3 vertex tile stages at
- * a time.  Shape 0: 960 records (FP32) / 640 (FP64), the default; shape 1:
- * 768 / 512.  Fewer records per chunk suit early, nearly uniform loads, more
- * suit clustered late loads (more tiles then fit in one chunk).  Both shapes
+/* Shape of the projection's tiles (Sec. 2.1, the particle-mesh
+ * projection): the number of vertices along z of the columns that a CTA
+ * marches through.  Shape 0, the default, follows from the mesh size; shape 1
+ * is half of it, which spreads a small or unevenly loaded mesh over more
+ * CTAs.  Both shapes
  * compute the same sums (only the order of additions inside a cell may
  * differ).  force 0 or 1 selects a shape; -2 keeps the current one; -1 times
  * the deposit of the context's current state with both shapes and keeps the

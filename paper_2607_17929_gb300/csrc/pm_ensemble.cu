@@ -76,7 +76,7 @@ void ens_join(pm_ensemble *e)
     }
 }
 
-// the batched step of the boxes: one deposit and one kick launch per precision (and deposit shape) over all
+// the batched step of the boxes: one deposit (per mode) and one kick launch per precision over all
 // boxes, the per-box transforms, solves and sorts on the k streams in between
 template <class T>
 void ens_particles(std::vector<pm::Ctx *> &cs, std::vector<pm::StepScalars> &ss, cudaStream_t st, bool deposit)
@@ -86,15 +86,15 @@ void ens_particles(std::vector<pm::Ctx *> &cs, std::vector<pm::StepScalars> &ss,
         pm::launch_kick_batch<T>(cs.data(), ss.data(), (int)cs.size(), st);
         return;
     }
-    for (int v = 0; v < 2; v++) {
+    for (const bool full : {true, false}) {
         std::vector<pm::Ctx *> cv;
         std::vector<pm::StepScalars> sv;
         for (size_t i = 0; i < cs.size(); i++)
-            if (cs[i]->dep_shape == v) {
+            if (cs[i]->newtonian != full) {
                 cv.push_back(cs[i]);
                 sv.push_back(ss[i]);
             }
-        if (!cv.empty()) pm::launch_project_batch<T>(cv.data(), sv.data(), (int)cv.size(), v, st);
+        if (!cv.empty()) pm::launch_project_batch<T>(cv.data(), sv.data(), (int)cv.size(), full, st);
     }
 }
 

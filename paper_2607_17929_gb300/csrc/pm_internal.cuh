@@ -94,7 +94,7 @@ struct Ctx {
     bool full_hc = false;       // PM_FULL_HC
     bool b_space = false;       // PM_B_SPACESPACE
     int col_shape[2] = {0, 0};  // shapes of the y and z column FFT passes (pm_fft_shapes)
-    int dep_shape = 0;          // record capacity of the deposit's shared-memory chunks (pm_deposit_shape)
+    int dep_shape = 0;          // column length of the deposit's tiles (pm_deposit_shape)
 
     // schedule (host, FP64)
     std::vector<double> a_n, dtau, a_half;
@@ -187,9 +187,9 @@ template <class T>
 void launch_solve(Ctx &c, const StepScalars &s);
 template <class T>
 void launch_kick_drift(Ctx &c, const StepScalars &s);
-// batched forms for the ensemble: one launch over n boxes of one precision (and one deposit shape)
+// batched forms for the ensemble: one launch over n boxes of one precision (all relativistic or all Newtonian)
 template <class T>
-void launch_project_batch(Ctx *const *cs, const StepScalars *ss, int n, int shape, cudaStream_t st);
+void launch_project_batch(Ctx *const *cs, const StepScalars *ss, int n, bool full, cudaStream_t st);
 template <class T>
 void launch_kick_batch(Ctx *const *cs, const StepScalars *ss, int n, cudaStream_t st);
 // times the deposit shapes on the context's current state and keeps the fastest (returns it)

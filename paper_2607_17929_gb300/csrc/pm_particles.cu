@@ -2,14 +2,17 @@
 // counting sort by cell, particle I/O.
 //
 // Projection (Sec. 2.1 "particle-mesh projection", Eqs. matterstress):
-// particles are kept sorted by cell.  One CTA owns an 8^3 tile of mesh
-// vertices and pulls every particle whose CIC cloud touches the tile (the
-// 9^3 cells [x0-1, x0+8)), computes its charges once into shared memory and
-// lets each thread accumulate the 9 source components of its own vertex in
-// registers.  No global atomics, and every mesh value is written once with
-// coalesced stores.  The same kernel assembles the configuration-space
-// sources of the field equations from phi_{n-1}, chi_{n-1}, phi_{n-2}.
+// particles are kept sorted by cell.  A CTA owns a column of mesh vertices and
+// marches along z, one cell plane at a time: a thread owns one cell of the
+// plane, adds the charges of its particles to the cell's 8 corners in
+// registers, and the corner sums of neighbouring cells meet in registers (z),
+// through a shuffle (x) and through shared memory (y).  No global atomics, and
+// every mesh value is written once.  The same kernel assembles the
+// configuration-space sources of the field equations from phi_{n-1},
+// chi_{n-1}, phi_{n-2}.
 #include <algorithm>
+#include <cmath>
+#include <type_traits>
 
 #include "pm_internal.cuh"
 
@@ -17,12 +20,6 @@ namespace pm {
 
 namespace {
 
-constexpr int TILE = 8;
-constexpr int REG = TILE + 1;        // 9 source cells per axis
-constexpr int FLD = TILE + 2;        // 10 field vertices per axis
-constexpr int NREG = REG * REG * REG;  // 729
-constexpr int NFLD = FLD * FLD * FLD;  // 1000
-constexpr int DEP_THREADS = TILE * TILE * TILE;  // 512
 constexpr int NK0SLOTS = 1024;
 
 // Per-cell accumulator of the T^00 charge, whose cell sums cancel against the
@@ -34,6 +31,7 @@ template <> struct Acc<double> {
     double s;
     __device__ __forceinline__ void zero() { s = 0.0; }
     __device__ __forceinline__ void add(double x) { s += x; }
+    __device__ __forceinline__ void add_product(double a, double b, double) { s = fma(a, b, s); }
     __device__ __forceinline__ double hi() const { return s; }
     __device__ __forceinline__ double lo() const { return 0.0; }
 };
@@ -48,6 +46,16 @@ template <> struct Acc<float> {
         s = t;
         c = __fadd_rn(c, e);
     }
+    // += a b.  The magic number M = 1.5 2^23 U rounds the product to a multiple of U, which sums up exactly in s
+    // below 2^24 U; the exact rest (at most U / 2) goes to c.  Five operations after the product instead of the
+    // seven of add().
+    __device__ __forceinline__ void add_product(float a, float b, float M)
+    {
+        const float x = __fmul_rn(a, b);
+        const float h = __fsub_rn(__fadd_rn(x, M), M);
+        s = __fadd_rn(s, h);
+        c = __fadd_rn(c, __fsub_rn(x, h));
+    }
     __device__ __forceinline__ float hi() const { return s; }
     __device__ __forceinline__ float lo() const { return c; }
 };
@@ -55,7 +63,7 @@ template <> struct Acc<float> {
 // 1 / sqrt(x) and a / b: the hardware approximations (a few ulp) in the mixed form, whose
 // FP32 rounding already sets the error; IEEE operations in FP64
 __device__ __forceinline__ float rsqrt_t(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double rsqrt_t(double x) { return 1.0 / sqrt(x); }
+__device__ __forceinline__ double rsqrt_t(double x) { return rsqrt(x); }
 __device__ __forceinline__ float div_t(float a, float b) { return __fdividef(a, b); }
 __device__ __forceinline__ double div_t(double a, double b) { return a / b; }
 
@@ -73,11 +81,14 @@ template <class T> struct DepParams {
     const T *phi2;   // phi_{n-2}
     Ptrs out;        // R, Fx, Fy, Fz, Sxx, Sxy, Sxz, Syy, Syz
     double *k0slots; // NK0SLOTS partial sums of the k = 0 excess
-    int N, nt;
-    int full;        // 1: relativistic sources; 0: R only (bootstrap / Newtonian)
-    int use_fields;  // phi/chi enter the charges (not in the bootstrap / Newtonian mode)
+    int N;
+    int nrow, ncol;  // vertices of a tile along x and y
+    int ntx, nty;    // tiles along x and y
+    int tz;          // vertices of a tile along z
+    int cyclic;      // one tile along x: the cell x0 - 1 is the row's last
     int newtonian;
     T a, a2, mass;
+    T magic;         // of Acc<float>::add_product: U = 2^-13 of a power of two above a particle's charge and the mean load
     T G;             // 4piG a^-2 N^3 (Newtonian: 4piG a^-1 N^3)
     T rb_hi, rb_lo;  // expected per-vertex charge sum of a uniform load, float-float split
     T c1, c2;        // 3Hc/dtau_{n-1}, 3Hc^2
@@ -106,27 +117,24 @@ template <class T> __device__ __forceinline__ T expm1_minus_x(T x)
     return s * x * x;
 }
 
-// Nonlinear remainder of Eq. fullHc at one vertex, from phi_{n-1} and chi_{n-1} staged with a halo of 1
-// (stride st[d] along axis d) and phi_{n-2}:
+// Nonlinear remainder of Eq. fullHc at one vertex from phi_{n-1} (ph, and its six neighbours up/dn along
+// each axis), chi_{n-1} (ch) and phi_{n-2}:
 //   Nl = (e^{2phi} - 1) Lap phi - 1/2 e^{2phi} |grad phi|^2
 //      + 3/2 [Hc^2 (e^x - 1 - x) - 2 Hc phi' (e^x - 1) + phi'^2 e^x],  x = -2 psi,
 // the bracket being (Hc - phi')^2 e^{-2psi} - Hc^2 + 2 Hc phi' + 2 Hc^2 psi regrouped so that no term
 // of size Hc^2 cancels.
 template <class T>
-__device__ __forceinline__ T hc_remainder(const T *sphi, const T *schi, int vo, const int (&st)[3], T phi2,
-                                          const DepParams<T> &p)
+__device__ __forceinline__ T hc_remainder(T ph, const T (&up)[3], const T (&dn)[3], T ch, T phi2, const DepParams<T> &p)
 {
-    const T ph = sphi[vo];
     T lap = T(-6) * ph, g2 = T(0);
 #pragma unroll
     for (int d = 0; d < 3; d++) {
-        const T up = sphi[vo + st[d]], dn = sphi[vo - st[d]];
-        lap += up + dn;
-        const T g = (up - dn) * p.halfN;
+        lap += up[d] + dn[d];
+        const T g = (up[d] - dn[d]) * p.halfN;
         g2 += g * g;
     }
     lap *= p.n2;
-    const T psi = ph - schi[vo];
+    const T psi = ph - ch;
     const T dphi = (ph - phi2) * p.inv_dt2;
     const T x = T(-2) * psi;
     const T em = expm1(x);
@@ -135,305 +143,564 @@ __device__ __forceinline__ T hc_remainder(const T *sphi, const T *schi, int vo, 
            T(1.5) * (p.hc * p.hc * expm1_minus_x(x) - T(2) * p.hc * dphi * em + dphi * dphi * (em + T(1)));
 }
 
-// Particle records per shared-memory chunk, the deposit's tunable "bin shape" (pm_deposit_shape): shape 0
-// (960 FP32) was the fastest of 640-1024 at 512^3 in early steps, shape 1 (768) is a little faster in the
-// first, unclustered steps and slower late.  Both keep three CTAs per SM in FP32.
-constexpr int NDEPSHAPES = 2;
-template <class T, int V> constexpr int dep_cap() { return sizeof(T) == 8 ? (V ? 512 : 640) : (V ? 768 : 960); }
+// ---------------------------------------------------------------------------
+// Mass deposit of the Newtonian mode in FP32: a particle's charge is its mass, so a vertex needs only the offsets
+// of its 8 cells' particles.  One CTA per 8^3 tile of vertices stages the offsets of the 9^3 cells [x0 - 1, x0 + 8)
+// in cell order, and each thread sums its vertex's products one by one with TwoSum, rows (z, y), (z, y - 1),
+// (z - 1, y), (z - 1, y - 1), cells x - 1 then x.  This order is kept: the force correction feeds R through BF16
+// layers, where a change in the last bit of R changes the momenta by 1e-3 of their size, so a faster summation
+// order (the columns below need 0.33 ms at 288^3 with 201^3 particles) is not taken here.
+// What bounds it: instruction issue of the 8 dependent sums per vertex.  256^3 with a particle per cell 0.51 ->
+// 0.35 ms, 288^3 with 201^3 particles at z = 2 0.65 -> 0.57, against the general tile kernel that staged whole charge
+// records and searched each particle's cell.
+// ---------------------------------------------------------------------------
+constexpr int MT = 8, MR = MT + 1, MCELLS = MR * MR * MR, MTHREADS = MT * MT * MT;
+constexpr int MCAP = 960;   // particles staged at a time (a nearly uniform load of one per cell has 729)
 
-template <class T, int V> size_t dep_smem()
-{
-    return sizeof(T) * (12 * dep_cap<T, V>() + 2 * NFLD) +
-           sizeof(int) * (3 * NREG + 64 + FLD * FLD + FLD);
-}
-
-// Per-particle record in shared memory: {fx, fy, fz, q00}, {q0x, q0y, q0z, Txx}, {Txy, Txz, Tyy, Tyz}
-// (trace-free T_ij, Tzz implied), read back with three 16-byte (FP32) or six 16-byte (FP64) loads.
-template <class T> struct alignas(16) DepRec {
-    T f[3], q00, q0[3], txx, txy, txz, tyy, tyz;
+struct MassSmem {
+    float4 rec[MCAP];                         // f
+    int off[MCELLS + 1];                      // exclusive scan of the cells' counts
+    int warp[MTHREADS / 32];
 };
-static_assert(sizeof(DepRec<float>) == 48 && sizeof(DepRec<double>) == 96, "packed record");
 
-// Exclusive scan of v[0..n) (n <= 2 * blockDim) in place; returns the total.
-__device__ int block_exclusive_scan(int *v, int n, int *warp_tmp)
+__device__ __forceinline__ void mass_tile(const DepParams<float> &p, const int b)
 {
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    int a = (2 * tid < n) ? v[2 * tid] : 0;
-    int b = (2 * tid + 1 < n) ? v[2 * tid + 1] : 0;
-    int s = a + b, x = s;
+    __shared__ MassSmem sm;
+    const int N = p.N, nt = N / MT, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int x0 = (b % nt) * MT, y0 = ((b / nt) % nt) * MT, z0 = (b / (nt * nt)) * MT;
+    // first particle and count of cells 2 tid and 2 tid + 1, then the exclusive scan of the counts
+    int n[2] = {0, 0}, s[2] = {0, 0};
+#pragma unroll
+    for (int q = 0; q < 2; q++) {
+        const int i = 2 * tid + q;
+        if (i < MCELLS) {
+            const int sx = i % MR, sy = (i / MR) % MR, sz = i / (MR * MR);
+            const int g = (wrapi(z0 - 1 + sz, N) * N + wrapi(y0 - 1 + sy, N)) * N + wrapi(x0 - 1 + sx, N);
+            s[q] = __ldg(p.start + g);
+            n[q] = __ldg(p.start + g + 1) - s[q];
+        }
+    }
+    int inc = n[0] + n[1];
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        int y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
+        const int v = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += v;
     }
-    if (lane == 31) warp_tmp[wid] = x;
+    if (lane == 31) sm.warp[wid] = inc;
     __syncthreads();
-    if (wid == 0) {
-        int nw = blockDim.x >> 5;
-        int w = lane < nw ? warp_tmp[lane] : 0, z = w;
+    int before = 0, total = 0;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            int y = __shfl_up_sync(0xffffffffu, z, o);
-            if (lane >= o) z += y;
-        }
-        if (lane < nw) warp_tmp[lane] = z - w;
-        if (lane == nw - 1) warp_tmp[32] = z;
+    for (int w = 0; w < MTHREADS / 32; w++) {
+        const int v = sm.warp[w];
+        before += w < wid ? v : 0;
+        total += v;
     }
-    __syncthreads();
-    int excl = warp_tmp[wid] + x - s;
-    if (2 * tid < n) v[2 * tid] = excl;
-    if (2 * tid + 1 < n) v[2 * tid + 1] = excl + a;
-    int total = warp_tmp[32];
-    __syncthreads();
-    return total;
-}
-
-// The deposit of one 8^3 vertex tile b of the box described by p (smem: dep_smem of this CAP).
-template <class T, int CAP>
-__device__ __forceinline__ void deposit_tile(const DepParams<T> &p, const int b)
-{
-    extern __shared__ __align__(16) unsigned char smem[];
-    DepRec<T> *rec = reinterpret_cast<DepRec<T> *>(smem);            // [CAP]
-    T *sphi = reinterpret_cast<T *>(rec + CAP);
-    T *schi = sphi + NFLD;
-    int *scnt = reinterpret_cast<int *>(schi + NFLD);
-    int *soff = scnt + NREG;
-    int *sgs = soff + NREG;
-    int *wtmp = sgs + NREG;                                          // 64 ints
-    int *rowb = wtmp + 64;                                           // [FLD*FLD] wrapped (z,y) row bases
-    int *xw = rowb + FLD * FLD;                                      // [FLD] wrapped x
-
-    const int N = p.N, nt = p.nt, tid = threadIdx.x;
-    const int x0 = (b % nt) * TILE, y0 = ((b / nt) % nt) * TILE, z0 = (b / (nt * nt)) * TILE;
-    if (tid < FLD * FLD) {
-        const int ry = tid % FLD, rz = tid / FLD;
-        rowb[tid] = (wrapi(z0 - 1 + rz, N) * N + wrapi(y0 - 1 + ry, N)) * N;
-    }
-    if (tid < FLD) xw[tid] = wrapi(x0 - 1 + tid, N);
+    const int e = before + inc - n[0] - n[1];
+    if (2 * tid <= MCELLS) sm.off[2 * tid] = e;
+    if (2 * tid + 1 <= MCELLS) sm.off[2 * tid + 1] = e + n[0];
     __syncthreads();
 
-    // potentials of the previous solve on the 10^3 vertices [x0-1, x0+8]
-    constexpr int NIT = (NFLD + DEP_THREADS - 1) / DEP_THREADS;
-    constexpr int RIT = (NREG + DEP_THREADS - 1) / DEP_THREADS;
-    T a[NIT], c[NIT];
-    int gs0[RIT], gs1[RIT];
-    if (p.use_fields) {
+    const int ox = tid % MT, oy = (tid / MT) % MT, oz = tid / (MT * MT);
+    Acc<float> acc;
+    acc.zero();
+    for (int lo = 0; lo < total; lo += MCAP) {
+        const int hi = min(total, lo + MCAP);
+        // each thread stages the particles of its two cells, two loads under way at a time
+        const int last = n[0] + n[1];
+        for (int k = max(lo - e, 0); k < min(last, hi - e); k += 2) {
+            float2 xy[2];
+            float z[2];
 #pragma unroll
-        for (int q = 0; q < NIT; q++) {
-            const int i = tid + q * DEP_THREADS;
-            if (i < NFLD) {
-                const int row = i / FLD, rx = i - row * FLD;
-                const int64_t g = (int64_t)rowb[row] + xw[rx];
-                a[q] = p.phi1[g];
-                c[q] = p.chi1[g];
-            }
-        }
-    }
-    // particle ranges of the 9^3 source cells [x0-1, x0+8)
-#pragma unroll
-    for (int q = 0; q < RIT; q++) {
-        const int i = tid + q * DEP_THREADS;
-        if (i < NREG) {
-            const int row = i / REG, sx = i - row * REG;
-            const int sy = row % REG, sz = row / REG;
-            const int64_t g = (int64_t)rowb[sy + FLD * sz] + xw[sx];
-            gs0[q] = p.start[g];
-            gs1[q] = p.start[g + 1];
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < NIT; q++) {
-        const int i = tid + q * DEP_THREADS;
-        if (i < NFLD) {
-            sphi[i] = p.use_fields ? a[q] : T(0);
-            schi[i] = p.use_fields ? c[q] : T(0);
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < RIT; q++) {
-        const int i = tid + q * DEP_THREADS;
-        if (i < NREG) {
-            scnt[i] = gs1[q] - gs0[q];
-            soff[i] = gs1[q] - gs0[q];
-            sgs[i] = gs0[q];
-        }
-    }
-    __syncthreads();
-    const int total = block_exclusive_scan(soff, NREG, wtmp);
-
-    const int ox = tid % TILE, oy = (tid / TILE) % TILE, oz = tid / (TILE * TILE);
-    Acc<T> acc00;
-    acc00.zero();
-    T acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    Acc<T> k0;   // this thread's share of the k = 0 excess (float-float in the mixed form)
-    k0.zero();
-    const bool full = p.full;
-
-    for (int lo = 0; lo < total; lo += CAP) {
-        const int hi = min(total, lo + CAP);
-        // source cell of local particle i: largest t with soff[t] <= i
-        auto cell_of = [&](int i) {
-            int t0 = 0, t1 = NREG - 1;
-            while (t0 < t1) {
-                int m = (t0 + t1 + 1) >> 1;
-                if (soff[m] <= i) t0 = m;
-                else t1 = m - 1;
-            }
-            return t0;
-        };
-        int tn = lo + tid < hi ? cell_of(lo + tid) : 0;
-        for (int i = lo + tid; i < hi; i += DEP_THREADS) {
-            const int t = tn;
-            if (i + DEP_THREADS < hi) {   // the next particle of this thread: its cell now, its record into L1
-                tn = cell_of(i + DEP_THREADS);
-                asm volatile("prefetch.global.L1 [%0];" ::"l"(p.part + sgs[tn] + (i + DEP_THREADS - soff[tn])));
-            }
-            const Particle<T> P = p.part[sgs[t] + (i - soff[t])];
-            const int sx = t % REG, sy = (t / REG) % REG, sz = t / (REG * REG);
-            DepRec<T> r;
-            r.f[0] = P.f[0];
-            r.f[1] = P.f[1];
-            r.f[2] = P.f[2];
-            if (!full && p.newtonian) {
-                r.q00 = p.mass;
-            } else {
-                T ph = 0, ch = 0;
-                if (p.use_fields) {
-                    const T fx = P.f[0], fy = P.f[1], fz = P.f[2];
-                    const T wx[2] = {T(1) - fx, fx}, wy[2] = {T(1) - fy, fy}, wz[2] = {T(1) - fz, fz};
-#pragma unroll
-                    for (int dz = 0; dz < 2; dz++)
-#pragma unroll
-                        for (int dy = 0; dy < 2; dy++)
-#pragma unroll
-                            for (int dx = 0; dx < 2; dx++) {
-                                const T w = wx[dx] * wy[dy] * wz[dz];
-                                const int v = (sx + dx) + FLD * ((sy + dy) + FLD * (sz + dz));
-                                ph += w * sphi[v];
-                                ch += w * schi[v];
-                            }
+            for (int j = 0; j < 2; j++)
+                if (k + j < last) {
+                    const float *q = reinterpret_cast<const float *>(p.part + (k + j < n[0] ? s[0] + k + j : s[1] + (k + j - n[0])));
+                    xy[j] = __ldg(reinterpret_cast<const float2 *>(q + 2));
+                    z[j] = __ldg(q + 4);
                 }
-                const T ux = P.u[0], uy = P.u[1], uz = P.u[2];
-                const T u2 = ux * ux + uy * uy + uz * uz;
-                const T e2 = p.a2 + u2;
-                const T iE = rsqrt_t(e2);
-                // E = a + u^2 / (E + a): the approximate E enters only the small term, so E keeps the
-                // accuracy of a (the T^00 charge cancels against the background in R)
-                const T dE = div_t(u2, e2 * iE + p.a);
-                const T E = p.a + dE;
-                const T v2 = u2 * iE * iE;
-                const T m = p.mass;
-                // T^00 charge and its excess over a particle at rest (k = 0 mode, summed in FP64)
-                r.q00 = m * E * (T(1) + T(3) * ph + ph * v2);
-                if (sx >= 1 && sy >= 1 && sz >= 1) k0.add(m * (dE + E * (T(3) * ph + ph * v2)));
-                if (full) {
-                    const T wv = m * (T(1) + T(4) * ph - ch);
-                    r.q0[0] = wv * ux;
-                    r.q0[1] = wv * uy;
-                    r.q0[2] = wv * uz;
-                    const T ws = m * (T(1) + T(3) * ph - ph * v2) * iE;
-                    const T txx = ws * ux * ux, tyy = ws * uy * uy, tzz = ws * uz * uz;
-                    const T tr3 = (txx + tyy + tzz) * T(1.0 / 3.0);
-                    r.txx = txx - tr3;
-                    r.txy = ws * ux * uy;
-                    r.txz = ws * ux * uz;
-                    r.tyy = tyy - tr3;
-                    r.tyz = ws * uy * uz;
-                }
-            }
-            rec[i - lo] = r;
+#pragma unroll
+            for (int j = 0; j < 2; j++)
+                if (k + j < last && e + k + j < hi) sm.rec[e + k + j - lo] = make_float4(xy[j].x, xy[j].y, z[j], 0.f);
         }
         __syncthreads();
-        // vertex o receives from source cells o - d, d in {0,1}^3, weight (d ? f : 1 - f) per axis.
-        // The two x-neighbours (region x = ox and ox + 1) are adjacent in the particle order.
+        // vertex o receives from cells o - d, d in {0,1}^3, weight (d ? f : 1 - f) per axis; the x-neighbours
+        // (region x = ox and ox + 1) are adjacent in the particle order
 #pragma unroll
         for (int dz = 0; dz < 2; dz++)
 #pragma unroll
             for (int dy = 0; dy < 2; dy++) {
-                const int ts = ox + REG * ((oy + 1 - dy) + REG * (oz + 1 - dz));  // cell with dx = 1
-                const int mid = soff[ts + 1];                                     // first particle with dx = 0
-                const int jb = max(soff[ts], lo), je = min(mid + scnt[ts + 1], hi);
-                for (int jj = jb; jj < je; jj++) {
-                    const DepRec<T> r = rec[jj - lo];
-                    const T wyz = (dy ? r.f[1] : T(1) - r.f[1]) * (dz ? r.f[2] : T(1) - r.f[2]);
-                    const T w = (jj < mid ? r.f[0] : T(1) - r.f[0]) * wyz;
-                    acc00.add(mulr(w, r.q00));
-                    if (full) {
-                        acc[0] += w * r.q0[0];
-                        acc[1] += w * r.q0[1];
-                        acc[2] += w * r.q0[2];
-                        acc[3] += w * r.txx;
-                        acc[4] += w * r.txy;
-                        acc[5] += w * r.txz;
-                        acc[6] += w * r.tyy;
-                        acc[7] += w * r.tyz;
-                    }
+                const int ts = ox + MR * ((oy + 1 - dy) + MR * (oz + 1 - dz));   // cell with dx = 1
+                const int mid = sm.off[ts + 1];                                  // first particle with dx = 0
+                const int je = min(sm.off[ts + 2], hi);
+                for (int j = max(sm.off[ts], lo); j < je; j++) {
+                    const float4 f = sm.rec[j - lo];
+                    const float wyz = (dy ? f.y : 1.f - f.y) * (dz ? f.z : 1.f - f.z);
+                    const float w = (j < mid ? f.x : 1.f - f.x) * wyz;
+                    acc.add(mulr(w, p.mass));
                 }
             }
         __syncthreads();
     }
+    const int go = ((z0 + oz) * N + (y0 + oy)) * N + (x0 + ox);
+    // the uniform background is removed before rounding
+    reinterpret_cast<float *>(p.out.p[0])[go] = p.G * ((acc.hi() - p.rb_hi) + (acc.lo() - p.rb_lo));
+}
 
-    const int64_t go = ((int64_t)(z0 + oz) * N + (y0 + oy)) * N + (x0 + ox);
-    const int vo = (ox + 1) + FLD * ((oy + 1) + FLD * (oz + 1));
-    const int st[3] = {1, FLD, FLD * FLD};
+__global__ void __launch_bounds__(MTHREADS, 4) k_mass(const __grid_constant__ DepParams<float> p) { mass_tile(p, blockIdx.x); }
+
+// ---------------------------------------------------------------------------
+// Deposit.  A CTA owns the vertices [x0, x0 + nrow) x [y0, y0 + ncol) x [z0, z0 + tz) and visits the cells
+// that reach them, one more in front along each axis, plane by plane along z.  Warp w takes the x-row of cells
+// y = y0 - 1 + w, whose particles are consecutive in memory:
+//  - lane i forms the weights and the 9 charges of the i-th particle of the row (32 at a time) and leaves them
+//    in shared memory, so that this work is even whatever the cells hold;
+//  - lane l, the vertex x0 + l, sums over the particles of the cells x - 1 and x, again consecutive, the shares
+//    of the row's four (y, z) corner lines: two of them belong to plane z, where the sums of the plane before
+//    wait in registers, and two to plane z + 1;
+//  - shared memory carries the y + 1 sums to the next row's warp, which then holds whole vertices.
+// What bounds it: instruction issue (FP32) and the FP64 pipe (FP64).  A particle's charges are formed once per
+// CTA that needs them (about 1.2 times: (nrow + 1)/nrow, (ncol + 1)/ncol and (tz + 1)/tz), its record is read
+// by two vertex lanes, and a vertex costs 36 products per particle of two cells.  Against 8^3 vertex tiles that
+// stage the charges of 9^3 cells and let each vertex gather from 8 cells (a record read 8 times, potentials, ranges
+// and a scan set up per tile), at 512^3 mixed 6.9 -> 4.0 ms early (sums of one plane in registers, 40 of them, so
+// 20 warps an SM), at 256^3 FP64 15.3 -> 8.8, late (192^3, z = 1, cells of up to 55 particles) 0.59 -> 0.56.  A cell per lane with its 8 corners in registers was faster early (3.4 ms) but ran as
+// long as its row's fullest cell (late 0.78 ms).
+// ---------------------------------------------------------------------------
+constexpr int DROWS = 10;                 // rows of cells of a tile along y, one warp each
+constexpr int DTY = DROWS - 1;            // and of vertices, at most
+constexpr int DEP_THREADS = 32 * DROWS;
+constexpr int DPX = 34, DPY = DTY + 2;    // staged potentials: x0 - 1 .. x0 + nrow, y0 - 1 .. y0 + ncol
+constexpr int DPN = DPX * DPY;
+constexpr int DRING = 5;                  // staged planes: z - 1 .. z + 2, and the one being fetched
+constexpr int NDEPSHAPES = 2;
+
+// sums exchanged per vertex: T00 (two words in FP32) and the other 8 charges
+template <class T, bool FULL> constexpr int dep_words() { return (sizeof(T) == 4 ? 2 : 1) + (FULL ? 8 : 0); }
+// words of a particle's weights and charges
+template <bool FULL> constexpr int dep_rec() { return FULL ? 17 : 9; }
+// staged particle records (the first 32 of a row, two planes), exchange rows (two planes), weights and charges,
+// staged potentials
+template <class T, bool FULL> constexpr size_t dep_smem()
+{
+    return 2 * DEP_THREADS * sizeof(Particle<T>) +
+           sizeof(T) * 32 * DROWS * (2 * dep_words<T, FULL>() + dep_rec<FULL>()) + sizeof(T) * (FULL ? 2 * DRING * DPN : 0);
+}
+
+// (hi, lo) += (h, l) of another sum, TwoSum on the high words
+template <class T> __device__ __forceinline__ void acc_merge(Acc<T> &s, const Acc<T> &o)
+{
+    s.add(o.hi());
+    if constexpr (sizeof(T) == 4) s.c += o.c;
+}
+// Cell, offset and momentum of one particle.
+template <class T> struct PartFU {
+    int cell;
+    T f[3], u[3];
+};
+// from its 16-byte parts, `step` parts apart
+__device__ __forceinline__ PartFU<float> unpack(const float4 *q, int step)
+{
+    const float4 a = q[0], b = q[step];
+    return {__float_as_int(a.x), {a.z, a.w, b.x}, {b.y, b.z, b.w}};
+}
+__device__ __forceinline__ PartFU<double> unpack(const double2 *q, int step)
+{
+    const double2 a = q[0], b = q[step], c = q[2 * step], d = q[3 * step];
+    return {__double2loint(a.x), {a.y, b.x, b.y}, {c.x, c.y, d.x}};
+}
+
+// Charges of one particle and its 8 CIC weights (w[4 dx + dy + 2 dz]).  lo/up: the staged potentials of the
+// cell's lower and upper plane at its corner (0, 0); chi DRING DPN values after phi.  ex receives the excess of the T^00 charge over a particle at rest (the k = 0 mode).
+template <class T, bool FULL>
+__device__ __forceinline__ void charges(const DepParams<T> &p, const PartFU<T> &P, const T *lo, const T *up, T (&w)[8],
+                                        T &q00, T (&q)[8], T &ex)
+{
+    const T fx = P.f[0], fy = P.f[1], fz = P.f[2];
+    const T gx = T(1) - fx, gy = T(1) - fy, gz = T(1) - fz;
+    const T yz[4] = {gy * gz, fy * gz, gy * fz, fy * fz};
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        w[i] = gx * yz[i];
+        w[4 + i] = fx * yz[i];
+    }
+    if (!FULL && p.newtonian) {
+        q00 = p.mass;
+        ex = T(0);
+        return;
+    }
+    T ph = 0, ch = 0;
+    if constexpr (FULL) {
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+            const T *s = (i & 2 ? up : lo) + (i >> 2) + (i & 1 ? DPX : 0);
+            ph += w[i] * s[0];
+            ch += w[i] * s[DRING * DPN];
+        }
+    }
+    const T ux = P.u[0], uy = P.u[1], uz = P.u[2];
+    const T u2 = ux * ux + uy * uy + uz * uz;
+    const T e2 = p.a2 + u2;
+    const T iE = rsqrt_t(e2);
+    // E = a + u^2 / (E + a): the approximate E enters only the small term, so E keeps the
+    // accuracy of a (the T^00 charge cancels against the background in R)
+    const T dE = div_t(u2, e2 * iE + p.a);
+    const T E = p.a + dE;
+    const T v2 = u2 * iE * iE;
+    const T m = p.mass;
+    const T mE = m * E, g = ph * (T(3) + v2);
+    q00 = mE + mE * g;
+    ex = m * dE + mE * g;
+    if constexpr (FULL) {
+        const T wv = m * (T(1) + T(4) * ph - ch);
+        q[0] = wv * ux;
+        q[1] = wv * uy;
+        q[2] = wv * uz;
+        const T ws = m * iE * (T(1) + ph * (T(3) - v2));
+        const T sx = ws * ux, sy = ws * uy;
+        const T tr3 = ws * u2 * T(1.0 / 3.0);
+        q[3] = sx * ux - tr3;
+        q[4] = sx * uy;
+        q[5] = sx * uz;
+        q[6] = sy * uy - tr3;
+        q[7] = sy * uz;
+    }
+}
+
+// sum over the warp, in every lane
+template <class T> __device__ __forceinline__ Acc<T> warp_sum(Acc<T> v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        Acc<T> b;
+        b.s = __shfl_xor_sync(0xffffffffu, v.s, o);
+        if constexpr (sizeof(T) == 4) b.c = __shfl_xor_sync(0xffffffffu, v.c, o);
+        acc_merge(v, b);
+    }
+    return v;
+}
+
+// values to and from 16-byte parts
+__device__ __forceinline__ float4 pack(const float *v) { return make_float4(v[0], v[1], v[2], v[3]); }
+__device__ __forceinline__ double2 pack(const double *v) { return make_double2(v[0], v[1]); }
+__device__ __forceinline__ void unpackv(const float4 &a, float *v)
+{
+    v[0] = a.x;
+    v[1] = a.y;
+    v[2] = a.z;
+    v[3] = a.w;
+}
+__device__ __forceinline__ void unpackv(const double2 &a, double *v)
+{
+    v[0] = a.x;
+    v[1] = a.y;
+}
+
+template <class T> __device__ __forceinline__ void cp_async_word(T *s, const T *g)
+{
+    const unsigned a = (unsigned)__cvta_generic_to_shared(s);
+    if constexpr (sizeof(T) == 4) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(a), "l"(g));
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(a), "l"(g));
+}
+
+// The field-equation sources of one vertex: dS the T^00 sum over the background, s the other 8 sums,
+// dn/md/up the staged potentials at the vertex in planes z - 1, z and z + 1.
+template <class T>
+__device__ __forceinline__ void dep_epilogue(const DepParams<T> &p, const T *dn, const T *md, const T *up, T phi2, T dS,
+                                             const T (&s)[8], int g, Acc<T> &k0)
+{
+    constexpr int CH = DRING * DPN;
+    const T ph = md[0], ch = md[CH];
+    const T pu[3] = {md[1], md[DPX], up[0]}, pd[3] = {md[-1], md[-DPX], dn[0]};
+    const T cu[3] = {md[CH + 1], md[CH + DPX], up[CH]}, cd[3] = {md[CH - 1], md[CH - DPX], dn[CH]};
     T nl = T(0);
     if (p.full_hc) {
-        nl = hc_remainder<T>(sphi, schi, vo, st, p.phi2[go], p);
+        nl = hc_remainder<T>(ph, pu, pd, ch, phi2, p);
         k0.add(-nl * (T)p.inv_g);   // the k = 0 mode carries the mean of -Nl
+    }
+    reinterpret_cast<T *>(p.out.p[0])[g] = p.G * dS - p.c1 * ph - p.c2 * ch - nl;
+    // with dp = 2 dx d phi, dc = 2 dx d chi and e = 2 dp - dc (of phi + psi = 2 phi - chi):
+    //   2 TF[2 d_i phi d_j phi - d_i(phi + psi) d_j(phi + psi)] = N^2/2 TF[2 dp_i dp_j - e_i e_j]
+    T dp[3], dc[3], e[3];
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+        dp[d] = pu[d] - pd[d];
+        dc[d] = cu[d] - cd[d];
+        e[d] = T(2) * dp[d] - dc[d];
+    }
+    if (p.write_f) {
+        const T f = (ph - phi2) * p.inv_dt2 * p.halfN;   // phi' / (2 dx)
+#pragma unroll
+        for (int d = 0; d < 3; d++) reinterpret_cast<T *>(p.out.p[1 + d])[g] = p.G * s[d] - f * (dp[d] - dc[d]);
+    }
+    const T G4 = T(4) * p.G, h = T(0.5) * p.n2;
+    auto quad = [&](int i, int j) { return T(2) * dp[i] * dp[j] - e[i] * e[j]; };
+    const T qxx = quad(0, 0), qyy = quad(1, 1), tr3 = (qxx + qyy + quad(2, 2)) * T(1.0 / 3.0);
+    reinterpret_cast<T *>(p.out.p[4])[g] = G4 * s[3] - h * (qxx - tr3);
+    reinterpret_cast<T *>(p.out.p[5])[g] = G4 * s[4] - h * quad(0, 1);
+    reinterpret_cast<T *>(p.out.p[6])[g] = G4 * s[5] - h * quad(0, 2);
+    reinterpret_cast<T *>(p.out.p[7])[g] = G4 * s[6] - h * (qyy - tr3);
+    reinterpret_cast<T *>(p.out.p[8])[g] = G4 * s[7] - h * quad(1, 2);
+}
+
+// A vertex lane's sums in one plane: of its own row of vertices and of the one at y + 1.
+template <class T> struct RowSums {
+    Acc<T> t00[2];
+    T q[2][8];
+    __device__ __forceinline__ void zero()
+    {
+#pragma unroll
+        for (int i = 0; i < 2; i++) {
+            t00[i].zero();
+#pragma unroll
+            for (int j = 0; j < 8; j++) q[i][j] = T(0);
+        }
+    }
+};
+
+// The particles of a warp's row of cells in one plane: those of the cell x0 - 1, then those of the others.
+// Particle i of the row is p.part[i < nh ? sh + i : sr + i]; a vertex lane's particles are prev .. end - 1, of
+// the cell at x - 1 below mid and of its own from there on.
+struct DepRow {
+    int sh, nh, sr, total;
+    int prev, mid, end;
+    int wrap;   // cyclic rows: lane 0's particles of the row's last cell are wrap .. total - 1
+};
+
+// A thread's view of its tile.
+template <class T, bool FULL> struct DepCol {
+    static constexpr int PQ = sizeof(Particle<T>) / 16;    // 16-byte parts of a record
+    static constexpr int VT = 16 / sizeof(T);              // values in 16 bytes
+    static constexpr int W = dep_words<T, FULL>(), R = dep_rec<FULL>();
+    using V = std::conditional_t<sizeof(T) == 4, float4, double2>;
+
+    const DepParams<T> &p;
+    V *stage;            // the row's first 32 records in this and the next plane, [par][part][thread]
+    T *xch, *rec, *ring;
+    int z0, nz, row;     // row: y N + x0
+    int nx;              // vertices of the row, 0 for a warp without one
+    int halo;            // index of the cell x0 - 1 relative to row
+    int go[2];           // staged potentials: where this thread's two entries of a plane come from (-1: none)
+    int sc;              // ring slot of plane z; plane z + i is in slot sc + i modulo DRING
+    Acc<T> k0;           // this thread's share of the k = 0 excess (float-float in the mixed form)
+
+    __device__ __forceinline__ int slot(int i) const { return sc + i >= DRING ? sc + i - DRING : sc + i; }
+    __device__ __forceinline__ void fetch(int slot, int z)
+    {
+        if constexpr (FULL) {
+            const int base = wrapi(z, p.N) * (p.N * p.N);
+            T *s = ring + slot * DPN + threadIdx.x;
+#pragma unroll
+            for (int q = 0; q < 2; q++)
+                if (go[q] >= 0) {
+                    cp_async_word(s + q * DEP_THREADS, p.phi1 + (base + go[q]));
+                    cp_async_word(s + q * DEP_THREADS + DRING * DPN, p.chi1 + (base + go[q]));
+                }
+        }
+    }
+    // the start and end of a lane's cell and of the cell x0 - 1
+    __device__ __forceinline__ int4 bounds(int z) const
+    {
+        if (nx == 0) return make_int4(0, 0, 0, 0);
+        const int32_t *c = p.start + (wrapi(z, p.N) * (p.N * p.N) + row);   // N^3 <= 2^30
+        const int l = min((int)threadIdx.x & 31, nx - 1);
+        return make_int4(__ldg(c + l), __ldg(c + l + 1), __ldg(c + halo), __ldg(c + halo + 1));
+    }
+    __device__ __forceinline__ DepRow range(const int4 &v) const
+    {
+        const int lane = threadIdx.x & 31;
+        DepRow r;
+        r.sh = v.z;
+        r.nh = p.cyclic ? 0 : v.w - v.z;
+        r.sr = __shfl_sync(0xffffffffu, v.x, 0) - r.nh;
+        r.total = __shfl_sync(0xffffffffu, v.y, 31) - r.sr;
+        r.mid = v.x - r.sr;
+        r.end = v.y - r.sr;
+        r.prev = __shfl_up_sync(0xffffffffu, r.mid, 1);
+        r.wrap = lane == 0 && p.cyclic ? v.z - r.sr : r.total;
+        if (lane == 0) r.prev = 0;
+        if (lane >= nx) r.prev = r.mid = r.end;   // nothing
+        return r;
+    }
+    // the row's first 32 records, into part `par` of the stage
+    __device__ __forceinline__ void fetch_row(int par, const DepRow &r)
+    {
+        const int i = threadIdx.x & 31;
+        if (i < r.total) {
+            const V *g = reinterpret_cast<const V *>(p.part + (i < r.nh ? r.sh + i : r.sr + i));
+#pragma unroll
+            for (int q = 0; q < PQ; q++) {
+                const unsigned a = (unsigned)__cvta_generic_to_shared(stage + (par * PQ + q) * DEP_THREADS + threadIdx.x);
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(a), "l"(g + q));
+            }
+        }
+    }
+
+    // One plane of cells, z = z0 + iz; PAR = iz & 1.  r: its rows, rn: those of the next plane (replaced by the
+    // ones after it).  A: the sums of plane z (on entry what the plane before put there), B: those of plane z + 1.
+    template <int PAR> __device__ __forceinline__ void plane(int iz, DepRow &r, DepRow &rn, RowSums<T> &A, RowSums<T> &B)
+    {
+        const int z = z0 + iz, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        const int cells = z * (p.N * p.N) + row;       // first cell of the row (used for 0 <= z < N)
+        const bool out = iz >= 0 && w > 0 && lane < nx;
+        const int col = w * DPX + lane + 1;            // the vertex in a staged plane
+        T f2 = 0;
+        if (FULL && out) f2 = __ldg(p.phi2 + cells + lane);
+        int4 nb = make_int4(0, 0, 0, 0);
+        if (iz + 2 < nz) nb = bounds(z + 2);
+        // this row's first records, copied since the plane before (the potentials fetched there may still be under way)
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        fetch_row(PAR ^ 1, rn);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        const T *lo = ring + sc * DPN + w * DPX, *up = ring + slot(1) * DPN + w * DPX;
+        B.zero();
+        V *rv = reinterpret_cast<V *>(rec);            // [part][32]: weights dx = 0, dx = 1, T00 and the other charges
+        const int base = wrapi(z, p.N) * (p.N * p.N) + row - 1;
+        for (int c0 = 0; c0 < r.total; c0 += 32) {
+            const int i = c0 + lane;
+            PartFU<T> P{};
+            int cx = 0;                                // the cell's lower corner in the row's staged potentials
+            if (i < r.total) {
+                if (c0 == 0) P = unpack(stage + PAR * PQ * DEP_THREADS + threadIdx.x, DEP_THREADS);
+                else P = unpack(reinterpret_cast<const V *>(p.part + (i < r.nh ? r.sh + i : r.sr + i)), 1);
+                if (i >= r.nh) cx = P.cell - base;
+            }
+            T wt[8], q00, q[8], ex;
+            charges<T, FULL>(p, P, lo + cx, up + cx, wt, q00, q, ex);
+            if (iz >= 0 && w > 0 && i >= r.nh && i < r.total) k0.add(ex);
+            __syncwarp();
+#pragma unroll
+            for (int k = 0; k < 8 / VT; k++) rv[32 * k + lane] = pack(wt + VT * k);
+            if constexpr (FULL) {
+#pragma unroll
+                for (int k = 0; k < 8 / VT; k++) rv[32 * (8 / VT + k) + lane] = pack(q + VT * k);
+            }
+            T *r0 = rec + 32 * (R - 1);
+            r0[lane] = q00;
+            __syncwarp();
+            // particles n0 .. n1 - 1 of the chunk, those below nm from the cell at x - 1
+            auto gather = [&](int n0, int n1, int nm) {
+#pragma unroll(FULL ? 1 : 2)
+                for (int n = n0; n < n1; n++) {
+                    T wn[4], qn[8];
+                    const V *v = rv + n + (n < nm ? 32 * (4 / VT) : 0);
+#pragma unroll
+                    for (int k = 0; k < 4 / VT; k++) unpackv(v[32 * k], wn + VT * k);
+                    const T t = r0[n];
+                    A.t00[0].add_product(wn[0], t, p.magic);
+                    A.t00[1].add_product(wn[1], t, p.magic);
+                    B.t00[0].add_product(wn[2], t, p.magic);
+                    B.t00[1].add_product(wn[3], t, p.magic);
+                    if constexpr (FULL) {
+#pragma unroll
+                        for (int k = 0; k < 8 / VT; k++) unpackv(rv[32 * (8 / VT + k) + n], qn + VT * k);
+#pragma unroll
+                        for (int j = 0; j < 8; j++) {
+                            A.q[0][j] += wn[0] * qn[j];
+                            A.q[1][j] += wn[1] * qn[j];
+                            B.q[0][j] += wn[2] * qn[j];
+                            B.q[1][j] += wn[3] * qn[j];
+                        }
+                    }
+                }
+            };
+            gather(max(r.prev - c0, 0), min(r.end - c0, 32), r.mid - c0);
+            if (p.cyclic) gather(max(r.wrap - c0, 0), min(r.total - c0, 32), 32);   // lane 0: the row's last cell
+            __syncwarp();
+        }
+        T *xo = xch + (PAR * DROWS + w) * (32 * W) + lane;
+        if (iz >= 0) {   // the sums for the row at y + 1
+            xo[0] = A.t00[1].hi();
+            if constexpr (sizeof(T) == 4) xo[32] = A.t00[1].lo();
+            if constexpr (FULL) {
+#pragma unroll
+                for (int j = 0; j < 8; j++) xo[(W - 8 + j) * 32] = A.q[1][j];
+            }
+        }
+        asm volatile("cp.async.wait_group 1;" ::: "memory");   // the potentials of plane z + 2
+        __syncthreads();
+        if (iz + 2 < nz) fetch(slot(3), z + 3);   // into the slot of plane z - 2, last read before the barrier
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        r = rn;
+        rn = range(nb);
+        if (out) {
+            const T *xi = xo - 32 * W;
+            // R: the uniform background a*Omega_m is removed before rounding
+            T dS = (A.t00[0].hi() + xi[0]) - p.rb_hi;
+            if constexpr (sizeof(T) == 4) dS += (A.t00[0].lo() + xi[32]) - p.rb_lo;
+            const int g = cells + lane;
+            if constexpr (!FULL) {
+                reinterpret_cast<T *>(p.out.p[0])[g] = p.G * dS;
+            } else {
+                T s[8];
+#pragma unroll
+                for (int j = 0; j < 8; j++) s[j] = A.q[0][j] + xi[(W - 8 + j) * 32];
+                dep_epilogue(p, ring + slot(DRING - 1) * DPN + col, ring + sc * DPN + col, ring + slot(1) * DPN + col, f2, dS,
+                             s, g, k0);
+            }
+        }
+        sc = slot(1);
+    }
+};
+
+// The deposit of tile b of the box described by p.
+template <class T, bool FULL>
+__device__ __forceinline__ void deposit_tile(const DepParams<T> &p, const int b)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int N = p.N, tid = threadIdx.x, w = tid >> 5;
+    using C = DepCol<T, FULL>;
+    C c{p};
+    c.stage = reinterpret_cast<typename C::V *>(smem);
+    c.rec = reinterpret_cast<T *>(smem + 2 * DEP_THREADS * sizeof(Particle<T>)) + w * (32 * C::R);
+    c.xch = reinterpret_cast<T *>(smem + 2 * DEP_THREADS * sizeof(Particle<T>)) + DROWS * (32 * C::R);
+    c.ring = c.xch + 2 * DROWS * (32 * C::W);              // phi, chi [DRING][DPN]
+    const int x0 = (b % p.ntx) * p.nrow, y0 = ((b / p.ntx) % p.nty) * p.ncol;
+    const int nx = min(p.nrow, N - x0), ny = min(p.ncol, N - y0);
+    c.z0 = (b / (p.ntx * p.nty)) * p.tz;
+    c.nz = min(p.tz, N - c.z0);
+    c.nx = w <= ny ? nx : 0;
+    c.row = (w <= ny ? wrapi(y0 - 1 + w, N) : 0) * N + x0;
+    c.halo = x0 > 0 ? -1 : N - 1;
+#pragma unroll
+    for (int q = 0; q < 2; q++) {   // entries tid and tid + DEP_THREADS of a plane (nx + 2 columns, ny + 2 rows used)
+        const int e = tid + q * DEP_THREADS;
+        const int ey = e / DPX, ex = e - ey * DPX;
+        c.go[q] = ey < ny + 2 && ex < nx + 2 ? wrapi(y0 - 1 + ey, N) * N + wrapi(x0 - 1 + ex, N) : -1;
+    }
+    static_assert(DPN <= 2 * DEP_THREADS, "two entries a thread");
+    // before the first plane of cells (z0 - 1): planes z0 - 1 .. z0 + 1 of the potentials and its first records
+    c.fetch(0, c.z0 - 1);
+    c.fetch(1, c.z0);
+    c.fetch(2, c.z0 + 1);
+    DepRow r = c.range(c.bounds(c.z0 - 1)), rn = c.range(c.bounds(c.z0));
+    c.fetch_row(1, r);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");   // an empty group: plane() leaves one pending
+    c.sc = 0;
+    c.k0.zero();
+    RowSums<T> A, B;
+    A.zero();
+    __syncthreads();
+    for (int iz = -1; iz < c.nz; iz += 2) {
+        c.template plane<1>(iz, r, rn, A, B);
+        if (iz + 1 == c.nz) break;
+        c.template plane<0>(iz + 1, r, rn, B, A);
     }
 
     // k = 0 excess: warp reduction of the (hi, lo) pairs with TwoSum, one FP64 atomic per warp into a slot
-    {
-        T hi = k0.hi(), lo = k0.lo();
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const T h2 = __shfl_down_sync(0xffffffffu, hi, o), l2 = __shfl_down_sync(0xffffffffu, lo, o);
-            const T t = hi + h2, bp = t - hi;
-            lo += l2 + ((hi - (t - bp)) + (h2 - bp));
-            hi = t;
-        }
-        if ((tid & 31) == 0 && !p.newtonian)
-            atomicAdd(&p.k0slots[(blockIdx.x * (DEP_THREADS >> 5) + (tid >> 5)) & (NK0SLOTS - 1)],
-                      (double)hi + (double)lo);
+    if (!p.newtonian) {
+        const Acc<T> k0 = warp_sum(c.k0);
+        if ((tid & 31) == 0)
+            atomicAdd(&p.k0slots[(blockIdx.x * DROWS + w) & (NK0SLOTS - 1)], (double)k0.hi() + (double)k0.lo());
     }
-
-    // epilogue: assemble the field-equation sources at vertex o
-    const T phc = sphi[vo], chc = schi[vo];
-    // R: the uniform background a*Omega_m is removed before rounding
-    const T dS = (acc00.hi() - p.rb_hi) + (acc00.lo() - p.rb_lo);
-    reinterpret_cast<T *>(p.out.p[0])[go] = p.G * dS - p.c1 * phc - p.c2 * chc - nl;
-    if (!full) return;
-    T gphi[3], gpsi[3];
-#pragma unroll
-    for (int d = 0; d < 3; d++) {
-        const T dp = (sphi[vo + st[d]] - sphi[vo - st[d]]) * p.halfN;
-        const T dc = (schi[vo + st[d]] - schi[vo - st[d]]) * p.halfN;
-        gphi[d] = dp;
-        gpsi[d] = dp - dc;
-    }
-    const T dphi = (phc - p.phi2[go]) * p.inv_dt2;
-    if (p.write_f) {
-#pragma unroll
-        for (int d = 0; d < 3; d++) reinterpret_cast<T *>(p.out.p[1 + d])[go] = p.G * acc[d] - dphi * gpsi[d];
-    }
-    T Q[3][3];
-#pragma unroll
-    for (int i = 0; i < 3; i++)
-#pragma unroll
-        for (int j = 0; j < 3; j++) Q[i][j] = T(2) * gphi[i] * gphi[j] - (gphi[i] + gpsi[i]) * (gphi[j] + gpsi[j]);
-    const T trQ3 = (Q[0][0] + Q[1][1] + Q[2][2]) * T(1.0 / 3.0);
-    const T G4 = T(4) * p.G;
-    reinterpret_cast<T *>(p.out.p[4])[go] = G4 * acc[3] - T(2) * (Q[0][0] - trQ3);
-    reinterpret_cast<T *>(p.out.p[5])[go] = G4 * acc[4] - T(2) * Q[0][1];
-    reinterpret_cast<T *>(p.out.p[6])[go] = G4 * acc[5] - T(2) * Q[0][2];
-    reinterpret_cast<T *>(p.out.p[7])[go] = G4 * acc[6] - T(2) * (Q[1][1] - trQ3);
-    reinterpret_cast<T *>(p.out.p[8])[go] = G4 * acc[7] - T(2) * Q[1][2];
 }
 
-template <class T, int V>
-__global__ void __launch_bounds__(DEP_THREADS, sizeof(T) == 4 ? 3 : 1) k_project(const __grid_constant__ DepParams<T> p)
+template <class T, bool FULL> constexpr int dep_ctas() { return sizeof(T) == 4 ? (FULL ? 2 : 3) : (FULL ? 1 : 2); }
+
+template <class T, bool FULL>
+__global__ void __launch_bounds__(DEP_THREADS, dep_ctas<T, FULL>()) k_project(const __grid_constant__ DepParams<T> p)
 {
-    deposit_tile<T, dep_cap<T, V>()>(p, blockIdx.x);
+    deposit_tile<T, FULL>(p, blockIdx.x);
 }
 
 // Several boxes in one launch (the batched ensemble): CTA j deposits tile j - first[i] of box i, the box whose
@@ -446,12 +713,19 @@ template <class T> struct DepBatch {
 };
 static_assert(sizeof(DepBatch<double>) < 32000, "kernel parameter space");
 
-template <class T, int V>
-__global__ void __launch_bounds__(DEP_THREADS, sizeof(T) == 4 ? 3 : 1) k_project_batch(const __grid_constant__ DepBatch<T> q)
+template <class T, bool FULL>
+__global__ void __launch_bounds__(DEP_THREADS, dep_ctas<T, FULL>()) k_project_batch(const __grid_constant__ DepBatch<T> q)
 {
     int i = 0;
     while (i + 1 < q.nbox && (int)blockIdx.x >= q.first[i + 1]) i++;
-    deposit_tile<T, dep_cap<T, V>()>(q.box[i], (int)blockIdx.x - q.first[i]);
+    deposit_tile<T, FULL>(q.box[i], (int)blockIdx.x - q.first[i]);
+}
+
+__global__ void __launch_bounds__(MTHREADS, 4) k_mass_batch(const __grid_constant__ DepBatch<float> q)
+{
+    int i = 0;
+    while (i + 1 < q.nbox && (int)blockIdx.x >= q.first[i + 1]) i++;
+    mass_tile(q.box[i], (int)blockIdx.x - q.first[i]);
 }
 
 // Sum the k = 0 slots: dscal[0] = sum over particles of the T^00 excess (block b: box b of a batch).
@@ -1113,6 +1387,34 @@ inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 }  // namespace
 
+// Tiles of the deposit.  Along x the vertices are split evenly over as few warps as hold them: 31, so that a row
+// of a nearly uniform load has 32 particles, or a whole row of up to 32, whose neighbour at x0 - 1 is its own last
+// cell.  Along z a tile of tz vertices visits tz + 1 planes of cells and takes about two more to start; tz makes
+// the number of waves times that smallest (64^3 mixed: 6, one wave, 17 us against 28 with one-plane tiles;
+// 512^3: 57; longer ones cost more in L2 than they save).  Shape 1 halves it.
+template <class T> void dep_tiles(DepParams<T> &p, bool full, int shape)
+{
+    const int N = p.N;
+    p.cyclic = N <= 32;
+    p.ntx = p.cyclic ? 1 : (N + 30) / 31;
+    p.nrow = (N + p.ntx - 1) / p.ntx;
+    p.nty = (N + DTY - 1) / DTY;
+    p.ncol = (N + p.nty - 1) / p.nty;
+    const int slots = 152 * (sizeof(T) == 4 ? (full ? dep_ctas<float, true>() : dep_ctas<float, false>())
+                                            : (full ? dep_ctas<double, true>() : dep_ctas<double, false>()));
+    int64_t best = INT64_MAX;
+    for (int tz = 1; tz <= std::min(N, 64); tz++) {
+        const int64_t waves = ((int64_t)p.ntx * p.nty * ((N + tz - 1) / tz) + slots - 1) / slots;
+        if (waves * (tz + 3) < best) {
+            best = waves * (tz + 3);
+            p.tz = tz;
+        }
+    }
+    if (shape == 1 && p.tz > 1) p.tz = (p.tz + 1) / 2;
+}
+
+inline bool dep_full(const StepScalars &s) { return !(s.newtonian || s.bootstrap); }
+
 template <class T> DepParams<T> dep_params(const Ctx &c, const StepScalars &s)
 {
     DepParams<T> p{};
@@ -1124,10 +1426,8 @@ template <class T> DepParams<T> dep_params(const Ctx &c, const StepScalars &s)
     for (int i = 0; i < 9; i++) p.out.p[i] = reinterpret_cast<T *>(c.src) + (size_t)i * c.nc;
     p.k0slots = c.dscal + 8;
     p.N = c.N;
-    p.nt = c.N / TILE;
     p.newtonian = s.newtonian;
-    p.full = !(s.newtonian || s.bootstrap);
-    p.use_fields = p.full;
+    dep_tiles(p, dep_full(s), c.dep_shape);
     p.a = (T)s.a;
     p.a2 = (T)(s.a * s.a);
     p.mass = (T)s.mass;
@@ -1142,6 +1442,8 @@ template <class T> DepParams<T> dep_params(const Ctx &c, const StepScalars &s)
     }
     p.rb_hi = (T)rb;
     p.rb_lo = (T)(rb - (double)p.rb_hi);
+    const double top = std::max(s.newtonian ? s.mass : s.a * s.mass, rb);   // sums stay exact up to 2048 of it
+    p.magic = (T)std::ldexp(1.5, std::ilogb(top) + 1 - 13 + 23);
     p.c1 = (T)s.c_phi_dt;
     p.c2 = (T)s.c_phi_h2;
     p.inv_dt2 = (T)s.inv_dtau_prev2;
@@ -1154,14 +1456,22 @@ template <class T> DepParams<T> dep_params(const Ctx &c, const StepScalars &s)
     return p;
 }
 
-template <class T, int V> void dep_attrs()
+template <class T, bool FULL> void dep_attrs()
 {
     static std::atomic<uint64_t> attr{0};
     if (first_on_device(attr)) {
-        cudaFuncSetAttribute(k_project<T, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dep_smem<T, V>());
-        cudaFuncSetAttribute(k_project_batch<T, V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)dep_smem<T, V>());
+        cudaFuncSetAttribute(k_project<T, FULL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dep_smem<T, FULL>());
+        if constexpr (sizeof(T) == 8 || FULL)
+            cudaFuncSetAttribute(k_project_batch<T, FULL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)dep_smem<T, FULL>());
     }
+}
+
+// the mixed Newtonian mode takes k_mass
+template <class T> bool dep_mass(const DepParams<T> &p) { return sizeof(T) == 4 && p.newtonian; }
+template <class T> int dep_ntiles(const DepParams<T> &p)
+{
+    return dep_mass(p) ? (p.N / MT) * (p.N / MT) * (p.N / MT) : p.ntx * p.nty * ((p.N + p.tz - 1) / p.tz);
 }
 
 template <class T>
@@ -1169,42 +1479,45 @@ void launch_project(Ctx &c, const StepScalars &s)
 {
     const DepParams<T> p = dep_params<T>(c, s);
     cudaMemsetAsync(c.dscal + 8, 0, sizeof(double) * NK0SLOTS, c.stream);
-    const int ntiles = (c.N / TILE) * (c.N / TILE) * (c.N / TILE);
-    if (c.dep_shape == 1) {
-        dep_attrs<T, 1>();
-        k_project<T, 1><<<ntiles, DEP_THREADS, dep_smem<T, 1>(), c.stream>>>(p);
-    } else {
-        dep_attrs<T, 0>();
-        k_project<T, 0><<<ntiles, DEP_THREADS, dep_smem<T, 0>(), c.stream>>>(p);
+    if (dep_full(s)) {
+        dep_attrs<T, true>();
+        k_project<T, true><<<dep_ntiles(p), DEP_THREADS, dep_smem<T, true>(), c.stream>>>(p);
+    } else if (!dep_mass(p)) {
+        dep_attrs<T, false>();
+        k_project<T, false><<<dep_ntiles(p), DEP_THREADS, dep_smem<T, false>(), c.stream>>>(p);
+    } else if constexpr (sizeof(T) == 4) {
+        k_mass<<<dep_ntiles(p), MTHREADS, 0, c.stream>>>(p);
     }
     k_k0_reduce<<<1, 1024, 0, c.stream>>>(c.dscal);
     c.launches += 2;
 }
 
-// One deposit launch over several boxes of one precision and one deposit shape (batches of MAXBATCH).
+// One deposit launch over several boxes of one precision, all relativistic or all Newtonian (batches of MAXBATCH).
 template <class T>
-void launch_project_batch(Ctx *const *cs, const StepScalars *ss, int n, int shape, cudaStream_t st)
+void launch_project_batch(Ctx *const *cs, const StepScalars *ss, int n, bool full, cudaStream_t st)
 {
     for (int b0 = 0; b0 < n; b0 += MAXBATCH) {
         const int nb = std::min(MAXBATCH, n - b0);
-        static DepBatch<T> q;   // host staging of the launch parameters (copied at launch)
+        thread_local DepBatch<T> q;   // host staging of the launch parameters (copied at launch)
         K0Batch kq{};
         q.nbox = nb;
         q.first[0] = 0;
         for (int i = 0; i < nb; i++) {
             Ctx &c = *cs[b0 + i];
             q.box[i] = dep_params<T>(c, ss[b0 + i]);
-            q.first[i + 1] = q.first[i] + (c.N / TILE) * (c.N / TILE) * (c.N / TILE);
+            q.first[i + 1] = q.first[i] + dep_ntiles(q.box[i]);
             kq.dscal[i] = c.dscal;
             cudaMemsetAsync(c.dscal + 8, 0, sizeof(double) * NK0SLOTS, st);
             c.launches += 2;
         }
-        if (shape == 1) {
-            dep_attrs<T, 1>();
-            k_project_batch<T, 1><<<q.first[nb], DEP_THREADS, dep_smem<T, 1>(), st>>>(q);
+        if (full) {
+            dep_attrs<T, true>();
+            k_project_batch<T, true><<<q.first[nb], DEP_THREADS, dep_smem<T, true>(), st>>>(q);
+        } else if constexpr (sizeof(T) == 4) {
+            k_mass_batch<<<q.first[nb], MTHREADS, 0, st>>>(q);
         } else {
-            dep_attrs<T, 0>();
-            k_project_batch<T, 0><<<q.first[nb], DEP_THREADS, dep_smem<T, 0>(), st>>>(q);
+            dep_attrs<T, false>();
+            k_project_batch<T, false><<<q.first[nb], DEP_THREADS, dep_smem<T, false>(), st>>>(q);
         }
         k_k0_reduce_batch<<<nb, 1024, 0, st>>>(kq);
     }
@@ -1262,7 +1575,7 @@ void launch_kick_batch(Ctx *const *cs, const StepScalars *ss, int n, cudaStream_
     kd_attrs<T>();
     for (int b0 = 0; b0 < n; b0 += MAXBATCH) {
         const int nb = std::min(MAXBATCH, n - b0);
-        static KdBatch<T> q;
+        thread_local KdBatch<T> q;
         q.nbox = nb;
         q.first[0] = 0;
         for (int i = 0; i < nb; i++) {
@@ -1417,7 +1730,7 @@ void launch_check_finite(Ctx &c, const double *d, int64_t n, int *d_flag)
 
 #define PM_INST(T)                                                                          \
     template void launch_project<T>(Ctx &, const StepScalars &);                            \
-    template void launch_project_batch<T>(Ctx *const *, const StepScalars *, int, int, cudaStream_t); \
+    template void launch_project_batch<T>(Ctx *const *, const StepScalars *, int, bool, cudaStream_t); \
     template void launch_kick_batch<T>(Ctx *const *, const StepScalars *, int, cudaStream_t); \
     template int tune_deposit_shape<T>(Ctx &, const StepScalars &);                         \
     template void launch_kick_drift<T>(Ctx &, const StepScalars &);                         \
