@@ -76,16 +76,12 @@ void ens_join(pm_ensemble *e)
     }
 }
 
-// the batched step of the boxes: one deposit (per mode) and one kick launch per precision over all
+// the batched step of the boxes: one deposit and one kick launch per precision and mode over all
 // boxes, the per-box transforms, solves and sorts on the k streams in between
 template <class T>
 void ens_particles(std::vector<pm::Ctx *> &cs, std::vector<pm::StepScalars> &ss, cudaStream_t st, bool deposit)
 {
     if (cs.empty()) return;
-    if (!deposit) {
-        pm::launch_kick_batch<T>(cs.data(), ss.data(), (int)cs.size(), st);
-        return;
-    }
     for (const bool full : {true, false}) {
         std::vector<pm::Ctx *> cv;
         std::vector<pm::StepScalars> sv;
@@ -94,7 +90,9 @@ void ens_particles(std::vector<pm::Ctx *> &cs, std::vector<pm::StepScalars> &ss,
                 cv.push_back(cs[i]);
                 sv.push_back(ss[i]);
             }
-        if (!cv.empty()) pm::launch_project_batch<T>(cv.data(), sv.data(), (int)cv.size(), full, st);
+        if (cv.empty()) continue;
+        if (deposit) pm::launch_project_batch<T>(cv.data(), sv.data(), (int)cv.size(), full, st);
+        else pm::launch_kick_batch<T>(cv.data(), sv.data(), (int)cv.size(), full, st);
     }
 }
 

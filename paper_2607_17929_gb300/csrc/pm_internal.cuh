@@ -191,7 +191,7 @@ void launch_kick_drift(Ctx &c, const StepScalars &s);
 template <class T>
 void launch_project_batch(Ctx *const *cs, const StepScalars *ss, int n, bool full, cudaStream_t st);
 template <class T>
-void launch_kick_batch(Ctx *const *cs, const StepScalars *ss, int n, cudaStream_t st);
+void launch_kick_batch(Ctx *const *cs, const StepScalars *ss, int n, bool full, cudaStream_t st);
 // times the deposit shapes on the context's current state and keeps the fastest (returns it)
 template <class T>
 int tune_deposit_shape(Ctx &c, const StepScalars &s);

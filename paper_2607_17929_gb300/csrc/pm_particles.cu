@@ -765,224 +765,289 @@ template <class T> struct KdParams {
     const int32_t *start;
     int32_t *count;
     const T *phi, *chi, *Bx, *By, *Bz;
-    int64_t np;
-    int N, nt;
-    int newtonian;
+    int N;
+    int nrow, ntx, tz;   // cells of a tile along x, tiles along x, cells along z
     T a, a2, a_half2, inv_a_half, dt_kick, dt_drift_N, halfN;
 };
 
-constexpr int KT = 8;                     // tile side in cells
-constexpr int KV = KT + 3;                // vertices per axis: x0-1 .. x0+9
-constexpr int KNV = KV * KV * KV;         // 1331
-constexpr int KD_THREADS = 256;
+// A CTA owns the cells [x0, x0 + nrow) x [y0, y0 + 8) x [z0, z0 + tz) and marches along z; warp w takes the row of
+// cells y0 + w, whose particles are consecutive in memory, one per lane.  The fields on the plane's vertices
+// [x0 - 1, x0 + nrow + 1] x [y0 - 1, y0 + 9] and the planes z - 1 .. z + 2 sit in a ring of five, one plane of which
+// is loaded while the warps work on the plane before.
+// What bounds it: the shared-memory pipe (a particle reads 32 vertices of 20 bytes, 5 of its 8 wavefronts) and, in
+// FP64, the FP64 pipe.  Against 8^3 tiles of 11^3 vertices, one search and three integer divisions per particle, and
+// the gradients of five fields kept in 20 registers (512^3 mixed 5.15 ms, 256^3 FP64 14.0, 288^3 Newtonian 0.52):
+// 3.6 ms, 11.1, 0.29.  Rows that hold more than 32 particles make their CTA's other warps wait (192^3 at z = 1:
+// 0.33 -> 0.33).  Two planes between barriers, records staged in shared memory instead of registers, four CTAs of 64
+// registers an SM, two of 128: 0.58, 0.48, 0.61, 0.52 ms against 0.46 at 256^3 (the first two take L1 from the loads).
+constexpr int KROWS = 8, KD_THREADS = 32 * KROWS;
+constexpr int KPX = 32 + 3, KPN = KPX * (KROWS + 3);   // vertices of a plane
+constexpr int KRING = 5;
+constexpr int KLD = (KPN + KD_THREADS - 1) / KD_THREADS;   // vertices of a plane per thread
 
 // phi, chi, B_x, B_y of one vertex in one 16-byte (FP32) or two 16-byte (FP64) loads
 template <class T> struct alignas(4 * sizeof(T) >= 16 ? 16 : 4 * sizeof(T)) Vtx4 {
     T phi, chi, bx, by;
 };
 
-template <class T> size_t kd_smem()
+template <class T, bool NEWT> constexpr size_t kd_smem()
 {
-    return sizeof(Vtx4<T>) * KNV + sizeof(T) * KNV + sizeof(int) * (KV * KV + KV + 2 * KT * KT + 2 + 33);
+    return KRING * KPN * sizeof(T) * (NEWT ? 1 : 5);
 }
 
-// Accumulate CIC value and centred-difference gradients of one vertex value s
-// at stencil offset (kx, ky, kz) in {0..3}^3 (offset -1 .. +2 from the cell);
-// terms whose weight is identically zero are skipped at compile time.
+// Accumulate the centred-difference gradient of one vertex value s at stencil offset (kx, ky, kz) in {0..3}^3
+// (offset -1 .. +2 from the cell); terms whose weight is identically zero are skipped at compile time.
 template <int kx, int ky, int kz, class T>
 __device__ __forceinline__ void stencil_acc(T s, const T *Wx, const T *Wy, const T *Wz, const T *Gx, const T *Gy,
-                                            const T *Gz, T &val, T (&g)[3])
+                                            const T *Gz, T (&g)[3])
 {
     constexpr bool cx = (kx == 1 || kx == 2), cy = (ky == 1 || ky == 2), cz = (kz == 1 || kz == 2);
-    if constexpr (cx && cy && cz) val += Wx[kx] * Wy[ky] * Wz[kz] * s;
     if constexpr (cy && cz) g[0] += Gx[kx] * (Wy[ky] * Wz[kz]) * s;
     if constexpr (cx && cz) g[1] += Gy[ky] * (Wx[kx] * Wz[kz]) * s;
     if constexpr (cx && cy) g[2] += Gz[kz] * (Wx[kx] * Wy[ky]) * s;
 }
 
+// Newtonian: the gradient of phi from the vertex planes pl[kz] (at stencil offset (0, 0)), vertex by vertex
 template <int I, class T>
-__device__ __forceinline__ void gather_all(const Vtx4<T> *sv, const T *sbz, int vb, bool newtonian, const T *Wx,
-                                           const T *Wy, const T *Wz, const T *Gx, const T *Gy, const T *Gz, T (&val)[5],
-                                           T (&grd)[5][3])
+__device__ __forceinline__ void gather_phi(const T *const (&pl)[4], const T *Wx, const T *Wy, const T *Wz, const T *Gx,
+                                           const T *Gy, const T *Gz, T (&g)[3])
 {
     if constexpr (I < 64) {
         constexpr int kx = I % 4, ky = (I / 4) % 4, kz = I / 16;
         constexpr bool cx = (kx == 1 || kx == 2), cy = (ky == 1 || ky == 2), cz = (kz == 1 || kz == 2);
-        if constexpr ((int)!cx + (int)!cy + (int)!cz <= 1) {
-            const int v = vb + kx + KV * (ky + KV * kz);
-            if (newtonian) {
-                stencil_acc<kx, ky, kz>(sv[v].phi, Wx, Wy, Wz, Gx, Gy, Gz, val[0], grd[0]);
-            } else {
-                const Vtx4<T> a = sv[v];
-                const T bz = sbz[v];
-                stencil_acc<kx, ky, kz>(a.phi, Wx, Wy, Wz, Gx, Gy, Gz, val[0], grd[0]);
-                stencil_acc<kx, ky, kz>(a.chi, Wx, Wy, Wz, Gx, Gy, Gz, val[1], grd[1]);
-                stencil_acc<kx, ky, kz>(a.bx, Wx, Wy, Wz, Gx, Gy, Gz, val[2], grd[2]);
-                stencil_acc<kx, ky, kz>(a.by, Wx, Wy, Wz, Gx, Gy, Gz, val[3], grd[3]);
-                stencil_acc<kx, ky, kz>(bz, Wx, Wy, Wz, Gx, Gy, Gz, val[4], grd[4]);
-            }
-        }
-        gather_all<I + 1>(sv, sbz, vb, newtonian, Wx, Wy, Wz, Gx, Gy, Gz, val, grd);
+        if constexpr ((int)!cx + (int)!cy + (int)!cz <= 1)
+            stencil_acc<kx, ky, kz>(pl[kz][kx + KPX * ky], Wx, Wy, Wz, Gx, Gy, Gz, g);
+        gather_phi<I + 1>(pl, Wx, Wy, Wz, Gx, Gy, Gz, g);
     }
 }
 
-// One CTA per 8^3 tile of cells: phi, chi and B on the 11^3 vertices around
-// the tile go to shared memory once; each thread then gathers the CIC value
-// and centred-difference gradients for one particle from there.
+// The relativistic gather.  The kick is minus the gradient of one scalar,
+//   s = (E + u^2/E) phi - E chi + u_j B_j      (coefficients c[5] of phi, chi, B of this particle),
+// so each of the 32 stencil vertices is first reduced to s (5 products) and only s is differenced and
+// interpolated, axis by axis (68 operations instead of the 280 of five fields' three gradients, and 3 sums
+// instead of 15).  g: 2 dx grad s; val: phi, chi, B at the particle.
 template <class T>
+__device__ __forceinline__ void gather_s(const Vtx4<T> *const (&sv)[4], const T *const (&sb)[4], const T (&c)[5], T fx, T fy,
+                                         T fz, T (&g)[3], T (&val)[5])
+{
+    const T gx = T(1) - fx, gy = T(1) - fy, gz = T(1) - fz;
+    // scalar at vertex (kx, ky) of plane kz; at the 8 corners of the cell the fields' values gather, too
+    auto at = [&](int kz, int v, T w, bool corner) {
+        const Vtx4<T> a = sv[kz][v];
+        const T b = sb[kz][v];
+        if (corner) {
+            val[0] += w * a.phi;
+            val[1] += w * a.chi;
+            val[2] += w * a.bx;
+            val[3] += w * a.by;
+            val[4] += w * b;
+        }
+        return c[0] * a.phi + c[1] * a.chi + (c[2] * a.bx + c[3] * a.by + c[4] * b);
+    };
+    auto line = [&](int kz, int v) {   // interpolated along x between kx = 1 and 2 (v: the vertex at kx = 1)
+        const T s1 = at(kz, v, T(0), false), s2 = at(kz, v + 1, T(0), false);
+        return s1 + fx * (s2 - s1);
+    };
+    T pz[4], px[2], py[2];   // per plane: s; its difference along x; along y
+#pragma unroll
+    for (int kz = 0; kz < 4; kz++) {
+        if (kz == 0 || kz == 3) {
+            const T v1 = line(kz, 1 + KPX), v2 = line(kz, 1 + 2 * KPX);
+            pz[kz] = v1 + fy * (v2 - v1);
+            continue;
+        }
+        const T wz = kz == 1 ? gz : fz;
+        T v[4], d[2];
+        v[0] = line(kz, 1);
+        v[3] = line(kz, 1 + 3 * KPX);
+#pragma unroll
+        for (int ky = 1; ky < 3; ky++) {
+            const T wyz = (ky == 1 ? gy : fy) * wz;
+            const T s0 = at(kz, KPX * ky, T(0), false), s1 = at(kz, KPX * ky + 1, gx * wyz, true),
+                    s2 = at(kz, KPX * ky + 2, fx * wyz, true), s3 = at(kz, KPX * ky + 3, T(0), false);
+            const T a = s2 - s0, b = s3 - s1;
+            v[ky] = s1 + fx * (s2 - s1);
+            d[ky - 1] = a + fx * (b - a);
+        }
+        pz[kz] = v[1] + fy * (v[2] - v[1]);
+        px[kz - 1] = d[0] + fy * (d[1] - d[0]);
+        const T a = v[2] - v[0], b = v[3] - v[1];
+        py[kz - 1] = a + fy * (b - a);
+    }
+    g[0] = px[0] + fz * (px[1] - px[0]);
+    g[1] = py[0] + fz * (py[1] - py[0]);
+    const T a = pz[2] - pz[0], b = pz[3] - pz[1];
+    g[2] = a + fz * (b - a);
+}
+
+template <class T, bool NEWT>
 __device__ __forceinline__ void kick_tile(const KdParams<T> &p, const int b)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    Vtx4<T> *sv = reinterpret_cast<Vtx4<T> *>(smem);              // [KNV]
-    T *sbz = reinterpret_cast<T *>(sv + KNV);                      // [KNV]
-    int *rowb = reinterpret_cast<int *>(sbz + KNV);                // [KV*KV] wrapped (z,y) row bases
-    int *xw = rowb + KV * KV;                                      // [KV] wrapped x
-    int *roff = xw + KV;                                           // 65 row offsets (+1 pad)
-    int *rgs = roff + KT * KT + 2;                                 // 64 global row starts
-    int *wtmp = rgs + KT * KT;                                     // 33
-    const int N = p.N, nt = p.nt, tid = threadIdx.x;
-    const int x0 = (b % nt) * KT, y0 = ((b / nt) % nt) * KT, z0 = (b / (nt * nt)) * KT;
+    constexpr int PQ = sizeof(Particle<T>) / 16;
+    using V = std::conditional_t<sizeof(T) == 4, float4, double2>;
+    T *ring = reinterpret_cast<T *>(smem);
+    Vtx4<T> *sv = reinterpret_cast<Vtx4<T> *>(ring);                           // [KRING][KPN]
+    T *sb = NEWT ? ring : ring + 4 * KRING * KPN;                              // B_z (Newtonian: phi) [KRING][KPN]
+    const int N = p.N, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int x0 = (b % p.ntx) * p.nrow, y0 = ((b / p.ntx) % (N / KROWS)) * KROWS, z0 = b / (p.ntx * (N / KROWS)) * p.tz;
+    const int nx = min(p.nrow, N - x0), nz = min(p.tz, N - z0);
+    const int row = (y0 + w) * N + x0;
 
-    if (tid < KV * KV) {
-        const int ry = tid % KV, rz = tid / KV;
-        rowb[tid] = (wrapi(z0 - 1 + rz, N) * N + wrapi(y0 - 1 + ry, N)) * N;
-    }
-    if (tid < KV) xw[tid] = wrapi(x0 - 1 + tid, N);
-    // particle rows of the tile: cells (x0 .. x0+7, y, z) are contiguous
-    int cnt = 0;
-    if (tid < KT * KT) {
-        const int ry = tid % KT, rz = tid / KT;
-        const int64_t c0 = ((int64_t)(z0 + rz) * N + (y0 + ry)) * N + x0;
-        const int gs = p.start[c0];
-        cnt = p.start[c0 + KT] - gs;
-        rgs[tid] = gs;
-    }
-    {
-        const int lane = tid & 31, wid = tid >> 5;
-        int x = cnt;
+    // this thread's vertices of a plane: where they come from (-1: none)
+    int go[KLD];
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (wid < 2 && lane == 31) wtmp[wid] = x;
-        __syncthreads();
-        if (tid < KT * KT) roff[tid] = x - cnt + (wid == 1 ? wtmp[0] : 0);
-        if (tid == 0) roff[KT * KT] = wtmp[0] + wtmp[1];
+    for (int q = 0; q < KLD; q++) {
+        const int e = tid + q * KD_THREADS, ey = e / KPX, ex = e - ey * KPX;
+        go[q] = e < KPN && ex < nx + 3 ? wrapi(y0 - 1 + ey, N) * N + wrapi(x0 - 1 + ex, N) : -1;
     }
-    // fields on the vertex block: every load of this thread's vertices issued before the stores
-    if (p.newtonian) {
-        for (int i = tid; i < KNV; i += KD_THREADS) {
-            const int row = i / KV, rx = i - row * KV;
-            Vtx4<T> a;
-            a.phi = __ldg(p.phi + (int64_t)rowb[row] + xw[rx]);
-            sv[i] = a;
-        }
-    } else {
-        constexpr int KIT = (KNV + KD_THREADS - 1) / KD_THREADS;
-        Vtx4<T> va[KIT];
-        T vz[KIT];
+    Vtx4<T> va[NEWT ? 1 : KLD];
+    T vb[KLD];
+    auto load = [&](int z) {
+        const int base = wrapi(z, N) * (N * N);
 #pragma unroll
-        for (int q = 0; q < KIT; q++) {
-            const int i = tid + q * KD_THREADS;
-            if (i < KNV) {
-                const int row = i / KV, rx = i - row * KV;
-                const int64_t g = (int64_t)rowb[row] + xw[rx];
-                va[q].phi = __ldg(p.phi + g);
-                va[q].chi = __ldg(p.chi + g);
-                va[q].bx = __ldg(p.Bx + g);
-                va[q].by = __ldg(p.By + g);
-                vz[q] = __ldg(p.Bz + g);
+        for (int q = 0; q < KLD; q++)
+            if (go[q] >= 0) {
+                const int g = base + go[q];
+                if constexpr (NEWT) {
+                    vb[q] = __ldg(p.phi + g);
+                } else {
+                    va[q].phi = __ldg(p.phi + g);
+                    va[q].chi = __ldg(p.chi + g);
+                    va[q].bx = __ldg(p.Bx + g);
+                    va[q].by = __ldg(p.By + g);
+                    vb[q] = __ldg(p.Bz + g);
+                }
             }
-        }
+    };
+    auto keep = [&](int slot) {
 #pragma unroll
-        for (int q = 0; q < KIT; q++) {
-            const int i = tid + q * KD_THREADS;
-            if (i < KNV) {
-                sv[i] = va[q];
-                sbz[i] = vz[q];
+        for (int q = 0; q < KLD; q++)
+            if (go[q] >= 0) {
+                if constexpr (!NEWT) sv[slot * KPN + tid + q * KD_THREADS] = va[q];
+                sb[slot * KPN + tid + q * KD_THREADS] = vb[q];
             }
+    };
+    // a row's first 32 records, ahead of their plane
+    V nxt[PQ];
+    auto fetch = [&](int s, int e) {
+        if (s + lane < e) {
+#pragma unroll
+            for (int q = 0; q < PQ; q++) nxt[q] = reinterpret_cast<const V *>(p.part + s + lane)[q];
         }
+    };
+    for (int i = 0; i < 4; i++) {   // planes z0 - 1 .. z0 + 2
+        load(z0 - 1 + i);
+        keep(i);
     }
+    const int32_t *st = p.start + z0 * (N * N) + row;
+    int s0 = __ldg(st), e0 = __ldg(st + nx), s1 = 0, e1 = 0;
+    if (nz > 1) {
+        s1 = __ldg(st + N * N);
+        e1 = __ldg(st + N * N + nx);
+    }
+    fetch(s0, e0);
     __syncthreads();
-    const int total = roff[KT * KT];
-    const T hn = p.halfN;
-    for (int i = tid; i < total; i += KD_THREADS) {
-        int r0 = 0, r1 = KT * KT - 1;
-        while (r0 < r1) {
-            const int m = (r0 + r1 + 1) >> 1;
-            if (roff[m] <= i) r0 = m;
-            else r1 = m - 1;
+
+    int sc = 0;   // slot of plane z - 1
+    for (int iz = 0; iz < nz; iz++) {
+        const int z = z0 + iz;
+        if (iz + 1 < nz) load(z + 3);
+        int s2 = 0, e2 = 0;
+        if (iz + 2 < nz) {
+            s2 = __ldg(st + (iz + 2) * (N * N));
+            e2 = __ldg(st + (iz + 2) * (N * N) + nx);
         }
-        const int64_t gi = (int64_t)rgs[r0] + (i - roff[r0]);
-        Particle<T> P = p.part[gi];
-        const int ix = P.cell % N, iy = (P.cell / N) % N, iz = P.cell / (N * N);
-        const int vb = (ix - x0) + KV * ((iy - y0) + KV * (iz - z0));  // vertex block index of offset -1
-        const T fx = P.f[0], fy = P.f[1], fz = P.f[2];
-        const T Wx[4] = {0, T(1) - fx, fx, 0}, Wy[4] = {0, T(1) - fy, fy, 0}, Wz[4] = {0, T(1) - fz, fz, 0};
-        const T Gx[4] = {-(T(1) - fx) * hn, -fx * hn, (T(1) - fx) * hn, fx * hn};
-        const T Gy[4] = {-(T(1) - fy) * hn, -fy * hn, (T(1) - fy) * hn, fy * hn};
-        const T Gz[4] = {-(T(1) - fz) * hn, -fz * hn, (T(1) - fz) * hn, fz * hn};
-        T val[5] = {0, 0, 0, 0, 0};
-        T grd[5][3] = {};
-        gather_all<0>(sv, sbz, vb, p.newtonian, Wx, Wy, Wz, Gx, Gy, Gz, val, grd);
-        T u[3] = {P.u[0], P.u[1], P.u[2]};
-        T dx[3];
-        if (p.newtonian) {
+        V rec[PQ];
 #pragma unroll
-            for (int d = 0; d < 3; d++) u[d] -= p.dt_kick * p.a * grd[0][d];
+        for (int q = 0; q < PQ; q++) rec[q] = nxt[q];
+        fetch(s1, e1);
+        const int base = z * (N * N) + row;
+        for (int i = s0 + lane; i < e0; i += 32) {
+            if (i >= s0 + 32) {
 #pragma unroll
-            for (int d = 0; d < 3; d++) dx[d] = p.dt_drift_N * u[d] * p.inv_a_half;
-        } else {
-            const T u2 = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-            const T e2 = p.a2 + u2;
-            const T iE = rsqrt_t(e2);
-            const T E = e2 * iE;
-            const T u2E = u2 * iE;
-            T K[3];
+                for (int q = 0; q < PQ; q++) rec[q] = reinterpret_cast<const V *>(p.part + i)[q];
+            }
+            Particle<T> P = *reinterpret_cast<const Particle<T> *>(rec);
+            const int cx = P.cell - base;
+            const int vo = w * KPX + cx;   // vertex at stencil offset (0, 0) in its plane
+            const T fx = P.f[0], fy = P.f[1], fz = P.f[2];
+            T u[3] = {P.u[0], P.u[1], P.u[2]};
+            T dx[3];
+            int slot[4];
+#pragma unroll
+            for (int k = 0; k < 4; k++) slot[k] = (sc + k >= KRING ? sc + k - KRING : sc + k) * KPN + vo;
+            const T *const pb[4] = {sb + slot[0], sb + slot[1], sb + slot[2], sb + slot[3]};
+            if constexpr (NEWT) {
+                const T hn = p.halfN;
+                const T Wx[4] = {0, T(1) - fx, fx, 0}, Wy[4] = {0, T(1) - fy, fy, 0}, Wz[4] = {0, T(1) - fz, fz, 0};
+                const T Gx[4] = {-(T(1) - fx) * hn, -fx * hn, (T(1) - fx) * hn, fx * hn};
+                const T Gy[4] = {-(T(1) - fy) * hn, -fy * hn, (T(1) - fy) * hn, fy * hn};
+                const T Gz[4] = {-(T(1) - fz) * hn, -fz * hn, (T(1) - fz) * hn, fz * hn};
+                T grd[3] = {0, 0, 0};
+                gather_phi<0>(pb, Wx, Wy, Wz, Gx, Gy, Gz, grd);
+#pragma unroll
+                for (int d = 0; d < 3; d++) u[d] -= p.dt_kick * p.a * grd[d];
+#pragma unroll
+                for (int d = 0; d < 3; d++) dx[d] = mulr(mulr(p.dt_drift_N, u[d]), p.inv_a_half);   // no FMA with the offset
+            } else {
+                const T u2 = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+                const T e2 = p.a2 + u2;
+                const T iE = rsqrt_t(e2);
+                const T E = e2 * iE;
+                const T c[5] = {E + u2 * iE, -E, u[0], u[1], u[2]};
+                const Vtx4<T> *const pv[4] = {sv + slot[0], sv + slot[1], sv + slot[2], sv + slot[3]};
+                T val[5] = {0, 0, 0, 0, 0}, g[3];
+                gather_s(pv, pb, c, fx, fy, fz, g, val);
+                const T dtk = p.dt_kick * p.halfN;
+#pragma unroll
+                for (int d = 0; d < 3; d++) u[d] -= dtk * g[d];
+                const T v2 = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+                const T iEd = rsqrt_t(p.a_half2 + v2);
+                const T fac = (T(1) + T(3) * val[0] - val[1] - val[0] * v2 * iEd * iEd) * iEd;
+#pragma unroll
+                for (int d = 0; d < 3; d++) dx[d] = p.dt_drift_N * (u[d] * fac + val[2 + d]);
+            }
+            const T fo[3] = {fx, fy, fz};
+            const int io[3] = {x0 + cx, y0 + w, z};
+            int inew[3];
 #pragma unroll
             for (int d = 0; d < 3; d++) {
-                const T dpsi = grd[0][d] - grd[1][d];
-                K[d] = -E * dpsi - u2E * grd[0][d] - (u[0] * grd[2][d] + u[1] * grd[3][d] + u[2] * grd[4][d]);
+                T f = fo[d] + dx[d];
+                T fl = floor(f);
+                f -= fl;
+                // a finite move is far below N cells; anything else (NaN, Inf) keeps the cell
+                int carry = (fabs(fl) < (T)N) ? (int)fl : 0;
+                if (f >= T(1)) {
+                    f = T(0);
+                    carry += 1;
+                }
+                inew[d] = wrapi(io[d] + carry, N);   // |carry| <= N
+                P.f[d] = f;
+                P.u[d] = u[d];
             }
-#pragma unroll
-            for (int d = 0; d < 3; d++) u[d] += p.dt_kick * K[d];
-            const T v2 = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-            const T iEd = rsqrt_t(p.a_half2 + v2);
-            const T fac = (T(1) + T(3) * val[0] - val[1] - val[0] * v2 * iEd * iEd) * iEd;
-#pragma unroll
-            for (int d = 0; d < 3; d++) dx[d] = p.dt_drift_N * (u[d] * fac + val[2 + d]);
+            P.cell = (inew[2] * N + inew[1]) * N + inew[0];
+            p.part[i] = P;
+            atomicAdd(&p.count[P.cell], 1);
         }
-        const T fo[3] = {fx, fy, fz};
-        const int io[3] = {ix, iy, iz};
-        int inew[3];
-#pragma unroll
-        for (int d = 0; d < 3; d++) {
-            T f = fo[d] + dx[d];
-            T fl = floor(f);
-            f -= fl;
-            // a finite move is far below N cells; anything else (NaN, Inf) keeps the cell
-            int carry = (fabs(fl) < (T)N) ? (int)fl : 0;
-            if (f >= T(1)) {
-                f = T(0);
-                carry += 1;
-            }
-            int c = (io[d] + carry) % N;
-            if (c < 0) c += N;
-            inew[d] = c;
-            P.f[d] = f;
-            P.u[d] = u[d];
-        }
-        P.cell = (inew[2] * N + inew[1]) * N + inew[0];
-        p.part[gi] = P;
-        atomicAdd(&p.count[P.cell], 1);
+        // plane z + 3 into the slot of plane z - 2, last read before the barrier of the plane before
+        if (iz + 1 < nz) keep(sc + 4 >= KRING ? sc + 4 - KRING : sc + 4);
+        __syncthreads();
+        sc = sc + 1 == KRING ? 0 : sc + 1;
+        s0 = s1;
+        e0 = e1;
+        s1 = s2;
+        e1 = e2;
     }
 }
 
-template <class T>
-__global__ void __launch_bounds__(KD_THREADS, sizeof(T) == 4 ? 4 : 1) k_kick_drift(const __grid_constant__ KdParams<T> p)
+// CTAs an SM holds: the relativistic FP32 kernel needs 80 registers, the Newtonian one 64, FP64 128
+template <class T, bool NEWT> constexpr int kd_ctas() { return sizeof(T) == 4 ? (NEWT ? 4 : 3) : 2; }
+
+template <class T, bool NEWT>
+__global__ void __launch_bounds__(KD_THREADS, kd_ctas<T, NEWT>()) k_kick_drift(const __grid_constant__ KdParams<T> p)
 {
-    kick_tile<T>(p, blockIdx.x);
+    kick_tile<T, NEWT>(p, blockIdx.x);
 }
 
 template <class T> struct KdBatch {
@@ -992,12 +1057,12 @@ template <class T> struct KdBatch {
 };
 static_assert(sizeof(KdBatch<double>) < 32000, "kernel parameter space");
 
-template <class T>
-__global__ void __launch_bounds__(KD_THREADS, sizeof(T) == 4 ? 4 : 1) k_kick_batch(const __grid_constant__ KdBatch<T> q)
+template <class T, bool NEWT>
+__global__ void __launch_bounds__(KD_THREADS, kd_ctas<T, NEWT>()) k_kick_batch(const __grid_constant__ KdBatch<T> q)
 {
     int i = 0;
     while (i + 1 < q.nbox && (int)blockIdx.x >= q.first[i + 1]) i++;
-    kick_tile<T>(q.box[i], (int)blockIdx.x - q.first[i]);
+    kick_tile<T, NEWT>(q.box[i], (int)blockIdx.x - q.first[i]);
 }
 
 // ---------------------------------------------------------------------------
@@ -1523,22 +1588,32 @@ void launch_project_batch(Ctx *const *cs, const StepScalars *ss, int n, bool ful
     }
 }
 
+// Tiles of the kick: rows of up to 32 cells, as long along z as makes the number of waves times (tz + 2) smallest
+// (the fields of three more planes are loaded than cells are visited).
 template <class T> KdParams<T> kd_params(const Ctx &c, const StepScalars &s)
 {
     KdParams<T> p{};
     p.part = reinterpret_cast<Particle<T> *>(c.part[c.cur]);
     p.start = c.start;
     p.count = c.count;
-    p.nt = c.N / KT;
     const T *B = reinterpret_cast<const T *>(c.B);
     p.phi = reinterpret_cast<const T *>(c.phi[c.iphi_new]);
     p.chi = reinterpret_cast<const T *>(c.chi);
     p.Bx = B;
     p.By = B + c.nc;
     p.Bz = B + 2 * c.nc;
-    p.np = c.np;
     p.N = c.N;
-    p.newtonian = s.newtonian;
+    p.ntx = (c.N + 31) / 32;
+    p.nrow = (c.N + p.ntx - 1) / p.ntx;
+    const int slots = 152 * kd_ctas<T, false>();
+    int64_t best = INT64_MAX;
+    for (int tz = 1; tz <= std::min(c.N, 64); tz++) {
+        const int64_t waves = ((int64_t)p.ntx * (c.N / KROWS) * ((c.N + tz - 1) / tz) + slots - 1) / slots;
+        if (waves * (tz + 2) < best) {
+            best = waves * (tz + 2);
+            p.tz = tz;
+        }
+    }
     p.a = (T)s.a;
     p.a2 = (T)(s.a * s.a);
     p.a_half2 = (T)(s.a_half * s.a_half);
@@ -1549,30 +1624,36 @@ template <class T> KdParams<T> kd_params(const Ctx &c, const StepScalars &s)
     return p;
 }
 
-template <class T> void kd_attrs()
+template <class T> int kd_ntiles(const KdParams<T> &p) { return p.ntx * (p.N / KROWS) * ((p.N + p.tz - 1) / p.tz); }
+
+template <class T, bool NEWT> void kd_attrs()
 {
     static std::atomic<uint64_t> attr{0};
     if (first_on_device(attr)) {
-        cudaFuncSetAttribute(k_kick_drift<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kd_smem<T>());
-        cudaFuncSetAttribute(k_kick_batch<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kd_smem<T>());
+        cudaFuncSetAttribute(k_kick_drift<T, NEWT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kd_smem<T, NEWT>());
+        cudaFuncSetAttribute(k_kick_batch<T, NEWT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kd_smem<T, NEWT>());
     }
 }
 
 template <class T>
 void launch_kick_drift(Ctx &c, const StepScalars &s)
 {
-    kd_attrs<T>();
     const KdParams<T> p = kd_params<T>(c, s);
-    const int ntiles = (c.N / KT) * (c.N / KT) * (c.N / KT);
-    k_kick_drift<T><<<ntiles, KD_THREADS, kd_smem<T>(), c.stream>>>(p);
+    if (s.newtonian) {
+        kd_attrs<T, true>();
+        k_kick_drift<T, true><<<kd_ntiles(p), KD_THREADS, kd_smem<T, true>(), c.stream>>>(p);
+    } else {
+        kd_attrs<T, false>();
+        k_kick_drift<T, false><<<kd_ntiles(p), KD_THREADS, kd_smem<T, false>(), c.stream>>>(p);
+    }
     c.launches++;
 }
 
-// One gather + kick + drift launch over several boxes of one precision (batches of MAXBATCH).
+// One gather + kick + drift launch over several boxes of one precision, all relativistic or all Newtonian (batches
+// of MAXBATCH).
 template <class T>
-void launch_kick_batch(Ctx *const *cs, const StepScalars *ss, int n, cudaStream_t st)
+void launch_kick_batch(Ctx *const *cs, const StepScalars *ss, int n, bool full, cudaStream_t st)
 {
-    kd_attrs<T>();
     for (int b0 = 0; b0 < n; b0 += MAXBATCH) {
         const int nb = std::min(MAXBATCH, n - b0);
         thread_local KdBatch<T> q;
@@ -1581,10 +1662,16 @@ void launch_kick_batch(Ctx *const *cs, const StepScalars *ss, int n, cudaStream_
         for (int i = 0; i < nb; i++) {
             Ctx &c = *cs[b0 + i];
             q.box[i] = kd_params<T>(c, ss[b0 + i]);
-            q.first[i + 1] = q.first[i] + (c.N / KT) * (c.N / KT) * (c.N / KT);
+            q.first[i + 1] = q.first[i] + kd_ntiles(q.box[i]);
             c.launches++;
         }
-        k_kick_batch<T><<<q.first[nb], KD_THREADS, kd_smem<T>(), st>>>(q);
+        if (full) {
+            kd_attrs<T, false>();
+            k_kick_batch<T, false><<<q.first[nb], KD_THREADS, kd_smem<T, false>(), st>>>(q);
+        } else {
+            kd_attrs<T, true>();
+            k_kick_batch<T, true><<<q.first[nb], KD_THREADS, kd_smem<T, true>(), st>>>(q);
+        }
     }
 }
 
@@ -1731,7 +1818,7 @@ void launch_check_finite(Ctx &c, const double *d, int64_t n, int *d_flag)
 #define PM_INST(T)                                                                          \
     template void launch_project<T>(Ctx &, const StepScalars &);                            \
     template void launch_project_batch<T>(Ctx *const *, const StepScalars *, int, bool, cudaStream_t); \
-    template void launch_kick_batch<T>(Ctx *const *, const StepScalars *, int, cudaStream_t); \
+    template void launch_kick_batch<T>(Ctx *const *, const StepScalars *, int, bool, cudaStream_t); \
     template int tune_deposit_shape<T>(Ctx &, const StepScalars &);                         \
     template void launch_kick_drift<T>(Ctx &, const StepScalars &);                         \
     template void launch_sort<T>(Ctx &);                                                    \
