@@ -1207,6 +1207,99 @@ __global__ void __launch_bounds__(256) k_scatter(const Particle<T> *in, Particle
 }
 
 // ---------------------------------------------------------------------------
+// f64 <-> f32 conversions, integer parts and fractions on the integer pipes.  The FP64 pipe, which also runs the
+// conversion instructions, takes 16 cycles a warp instruction here: with them the load spent 1.02 ms on
+// 256^3 particles and the store 0.46, with these 0.23 and 0.21 (the bytes take 0.20).  Every result is the one of
+// the FP64 instructions, rounded to nearest even; what is not in the common range takes those, out of line, since
+// the compiler would otherwise run both and select.
+// ---------------------------------------------------------------------------
+__device__ __noinline__ float f64_to_f32_any(double d) { return (float)d; }
+__device__ __noinline__ double f32_to_f64_any(float f) { return (double)f; }
+__device__ __noinline__ double position_any(int c, float f, double inv_n) { return ((double)c + (double)f) * inv_n; }
+__device__ __noinline__ double wrap_unit(double x)
+{
+    if (!isfinite(x)) x = 0.0;   // keeps the cell index valid; the caller rejects the input
+    x -= floor(x);
+    return x >= 1.0 ? 0.0 : x;
+}
+
+__device__ __forceinline__ float f64_to_f32(double d)
+{
+    const uint64_t b = (uint64_t)__double_as_longlong(d), m = b & 0x7fffffffffffffffull;
+    const uint32_t sign = (uint32_t)(b >> 32) & 0x80000000u, e = (uint32_t)(m >> 52);
+    if (e - 897u < 253u)   // a normal float, also after rounding
+        return __uint_as_float(sign | ((uint32_t)((m + 0x0fffffffull + ((m >> 29) & 1)) >> 29) - (896u << 23)));
+    return e == 0 ? __uint_as_float(sign) : f64_to_f32_any(d);
+}
+__device__ __forceinline__ double f32_to_f64(float f)
+{
+    const uint32_t b = __float_as_uint(f), e = (b >> 23) & 255;
+    if (e - 1u < 254u)   // normal
+        return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
+    return (b << 1) == 0 ? __hiloint2double((int)b, 0) : f32_to_f64_any(f);
+}
+
+// Integer part (returned) and fraction of s in [0, 2^10].
+__device__ __forceinline__ int split(double s, double &f)
+{
+    const uint64_t b = (uint64_t)__double_as_longlong(s);
+    const int e = (int)(b >> 52) - 1023;
+    if (e < 0) {
+        f = s;
+        return 0;
+    }
+    const uint64_t m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
+    const uint64_t r = m & ((0x10000000000000ull >> e) - 1);   // the fraction is r 2^(e - 52)
+    f = 0.0;
+    if (r) {
+        const int lead = __clzll((long long)r) - 11;           // its exponent is e - lead
+        f = __longlong_as_double((long long)(((uint64_t)(e - lead + 1022) << 52) + (r << lead)));
+    }
+    return (int)(m >> (52 - e));
+}
+__device__ __forceinline__ int split(double s, float &f)
+{
+    const uint64_t b = (uint64_t)__double_as_longlong(s);
+    const int e = (int)(b >> 52) - 1023;
+    if (e < 0) {
+        f = f64_to_f32(s);
+        return 0;
+    }
+    const uint64_t m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
+    const int c = (int)(m >> (52 - e));
+    const uint64_t r = m & ((0x10000000000000ull >> e) - 1);   // the fraction is r 2^(e - 52)
+    f = 0.f;
+    if (r) {
+        const int top = 63 - __clzll((long long)r), x = top + e - 52;   // its exponent, -52 .. -1
+        const uint64_t v = r << (63 - top);   // leading bit at 63; 24 bits kept, ties to even
+        const uint64_t q = (v + 0x7fffffffffull + ((v >> 40) & 1));
+        // a carry out of bit 63 is the next power of two, whose mantissa is zero
+        const uint32_t mant = q < v ? 0x1000000u : (uint32_t)(q >> 40);
+        f = __uint_as_float(((uint32_t)(x + 126) << 23) + mant);
+    }
+    return c;
+}
+
+// (c + f) / N of a cell index below 2^10 and an offset in [0, 1); inv_n = 1 / N, scaled = 2^-42 / N
+__device__ __forceinline__ double position(int c, double f, double inv_n, double) { return ((double)c + f) * inv_n; }
+__device__ __forceinline__ double position(int c, float f, double inv_n, double scaled)
+{
+    const uint32_t b = __float_as_uint(f), e = b >> 23;
+    if (e - 108u < 19u || b == 0) {   // f = 0 or in [2^-19, 1): a multiple of 2^-42, so 2^42 (c + f) is one below 2^52
+        const uint64_t m = b == 0 ? 0 : (uint64_t)((b & 0x7fffffu) | 0x800000u) << (e - 108u);
+        const uint64_t n = ((uint64_t)c << 42) | m;
+        return (__longlong_as_double((long long)(0x4330000000000000ull | n)) - 4503599627370496.0) * scaled;
+    }
+    return position_any(c, f, inv_n);
+}
+
+// the two conversions above where the particle type is f32
+__device__ __forceinline__ void narrow(double d, float &f) { f = f64_to_f32(d); }
+__device__ __forceinline__ void narrow(double d, double &f) { f = d; }
+__device__ __forceinline__ double widen(float f) { return f32_to_f64(f); }
+__device__ __forceinline__ double widen(double f) { return f; }
+
+// ---------------------------------------------------------------------------
 // Particle I/O: f64 (x, y, z) rows <-> cell + offset records.
 // ---------------------------------------------------------------------------
 template <class T>
@@ -1222,22 +1315,17 @@ __global__ void k_load(const double *pos, const double *mom, int64_t first, int6
     for (int d = 0; d < 3; d++) {
         double x = pos[3 * k + d];
         const double u = mom[3 * k + d];
-        bad |= !isfinite(x) || !isfinite(u);
-        if (!isfinite(x)) x = 0.0;   // keeps the cell index valid; the caller rejects the input
-        x -= floor(x);
-        if (x >= 1.0) x = 0.0;
-        double s = x * N;
-        double fl = floor(s);
-        int c = (int)fl;
-        double f = s - fl;
+        const uint32_t xh = (uint32_t)__double2hiint(x);
+        bad |= (xh & 0x7ff00000u) == 0x7ff00000u || ((uint32_t)__double2hiint(u) & 0x7ff00000u) == 0x7ff00000u;
+        if (xh >= 0x3ff00000u) x = wrap_unit(x);   // not in [0, 1)
+        int c = split(x * N, P.f[d]);
         if (c >= N) c -= N;
         ic[d] = c;
-        P.f[d] = (T)f;
-        if (P.f[d] >= T(1)) {  // rounding of f to the storage type
+        if (P.f[d] >= T(1)) {  // rounding of the offset to the storage type
             P.f[d] = T(0);
-            ic[d] = (c + 1) % N;
+            ic[d] = c + 1 == N ? 0 : c + 1;
         }
-        P.u[d] = (T)u;
+        narrow(u, P.u[d]);
     }
     if (bad) *nonfinite = 1;
     P.cell = (ic[2] * N + ic[1]) * N + ic[0];
@@ -1371,7 +1459,7 @@ __global__ void k_unpermute(const Particle<T> *in, Particle<T> *out, int64_t np)
 constexpr int ST_P = 512;
 template <class T>
 __global__ void __launch_bounds__(256) k_store(const Particle<T> *byid, int64_t first, int64_t cnt, int N,
-                                               double inv_n, double *pos, double *mom, int vec)
+                                               double inv_n, double scaled, double *pos, double *mom, int vec)
 {
     __shared__ double sp[3 * ST_P], su[3 * ST_P];
     const int64_t base = (int64_t)blockIdx.x * ST_P;
@@ -1381,8 +1469,8 @@ __global__ void __launch_bounds__(256) k_store(const Particle<T> *byid, int64_t 
         const int ic[3] = {P.cell % N, (P.cell / N) % N, P.cell / (N * N)};
 #pragma unroll
         for (int d = 0; d < 3; d++) {
-            sp[3 * j + d] = ((double)ic[d] + (double)P.f[d]) * inv_n;
-            su[3 * j + d] = (double)P.u[d];
+            sp[3 * j + d] = position(ic[d], P.f[d], inv_n, scaled);
+            su[3 * j + d] = widen(P.u[d]);
         }
     }
     __syncthreads();
@@ -1432,8 +1520,15 @@ __global__ void k_density_fin(const double *rho, int64_t n, T *out)
 
 template <class T> __global__ void k_to_f64(const T *s, double *d, int64_t n)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) d[i] = (double)s[i];
+    // four values a thread: with one, starting the blocks takes longer than the copy
+    const int64_t i = (int64_t)blockIdx.x * (4 * 256) + threadIdx.x;
+    T v[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++)
+        if (i + 256 * k < n) v[k] = s[i + 256 * k];
+#pragma unroll
+    for (int k = 0; k < 4; k++)
+        if (i + 256 * k < n) d[i + 256 * k] = widen(v[k]);
 }
 
 template <class T> __global__ void k_from_f64(const double *s, T *d, int64_t n)
@@ -1755,7 +1850,8 @@ void launch_store_particles(Ctx &c, double *d_pos, double *d_mom, int64_t first,
     // 16-byte stores need 16-byte aligned arrays (the block offsets are multiples of 3 * 512 doubles)
     const int vec = ((reinterpret_cast<uintptr_t>(d_pos) | reinterpret_cast<uintptr_t>(d_mom)) & 15) == 0;
     k_store<T><<<nblk(count, ST_P), 256, 0, c.stream>>>(reinterpret_cast<const Particle<T> *>(c.part[o]), first,
-                                                        count, c.N, 1.0 / (double)c.N, d_pos, d_mom, vec);
+                                                        count, c.N, 1.0 / (double)c.N,
+                                                        std::ldexp(1.0 / (double)c.N, -42), d_pos, d_mom, vec);
 }
 
 void launch_load_packed(Ctx &c, const pm_packed_particle *in, int64_t first, int64_t count, int *d_bad)
@@ -1800,7 +1896,7 @@ void launch_density(Ctx &c, void *real_out)
 template <class T>
 void launch_to_f64(Ctx &c, const void *src, double *dst, int64_t n)
 {
-    k_to_f64<T><<<nblk(n, 256), 256, 0, c.stream>>>(reinterpret_cast<const T *>(src), dst, n);
+    k_to_f64<T><<<nblk(n, 4 * 256), 256, 0, c.stream>>>(reinterpret_cast<const T *>(src), dst, n);
 }
 
 template <class T>
