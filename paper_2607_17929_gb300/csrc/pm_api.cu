@@ -681,7 +681,6 @@ pm_status pm_init(const pm_config *cfg, pm_ctx **out)
     c.h0 = cfg->box_mpch / 2997.92458;
     c.four_pi_g = 1.5 * c.h0 * c.h0;
     c.mass = cfg->omega_m / (double)c.np;
-    c.plan = make_plan(c.N);
     // schedule
     {
         const Background bg(cfg->omega_m, c.h0);
@@ -719,10 +718,10 @@ pm_status pm_init(const pm_config *cfg, pm_ctx **out)
         {&c.spec, 9 * 2 * ts * (size_t)c.nh},
         {&c.tens, 4 * 2 * ts * (size_t)c.nh},
         {&c.ktab, ts * (size_t)c.N},
-        {&c.tw, 2 * ts * (size_t)c.N},
         {&c.tw2, 2 * ts * (size_t)(2 * c.N + 64)},
         {(void **)&c.dscal, sizeof(double) * (8 + 1024)},
         {&c.stage_buf, sizeof(double) * (size_t)c.stage_elems},
+        {&c.bstate, c.b_space ? 3 * 2 * ts * (size_t)c.nh : 0},   // 0: not needed
     };
     // PM_TEST_FAIL_ALLOC=k (test hook): the k-th device allocation of this call reports failure, to
     // exercise the clean-up path without exhausting the device
@@ -730,27 +729,19 @@ pm_status pm_init(const pm_config *cfg, pm_ctx **out)
     const int fail_at = fail_env ? std::atoi(fail_env) : 0;
     int nalloc = 0;
     for (const A &a : allocs) {
-        if (++nalloc == fail_at || cudaMalloc(a.p, a.bytes) != cudaSuccess) {
+        if (++nalloc == fail_at || (a.bytes > 0 && cudaMalloc(a.p, a.bytes) != cudaSuccess)) {
             cudaGetLastError();
             pm_destroy(ctx);
             return PM_ERR_OOM;
         }
     }
-    if (c.b_space && cudaMalloc(&c.bstate, 3 * 2 * ts * (size_t)c.nh) != cudaSuccess) {
-        cudaGetLastError();
-        c.bstate = nullptr;
-        pm_destroy(ctx);
-        return PM_ERR_OOM;
-    }
-    // tables: ktilde(i) = 2N sin(pi n_i / N), twiddles exp(-2 pi i k / N) (long double on the host)
+    // tables: ktilde(i) = 2N sin(pi n_i / N), the FFT stages' twiddles (long double on the host)
     {
-        std::vector<double> kt(c.N), tw(2 * c.N);
+        std::vector<double> kt(c.N);
         const long double pi = 3.141592653589793238462643383279502884L;
         for (int i = 0; i < c.N; i++) {
             const int m = i <= c.N / 2 ? i : i - c.N;
             kt[i] = (double)(2.0L * c.N * sinl(pi * m / c.N));
-            tw[2 * i] = (double)cosl(2.0L * pi * i / c.N);
-            tw[2 * i + 1] = (double)(-sinl(2.0L * pi * i / c.N));
         }
         std::vector<double> tw2;
         fast_twiddles(c.N, tw2);
@@ -762,18 +753,14 @@ pm_status pm_init(const pm_config *cfg, pm_ctx **out)
             cudaMemcpy(c.tw2, tw2.data(), sizeof(double) * tw2.size(), cudaMemcpyHostToDevice);
         }
         if (c.mixed) {
-            std::vector<float> ktf(kt.begin(), kt.end()), twf(tw.begin(), tw.end());
+            std::vector<float> ktf(kt.begin(), kt.end());
             for (int i = 0; i < c.N; i++) {
                 const int m = i <= c.N / 2 ? i : i - c.N;
                 ktf[i] = (float)(2.0L * c.N * sinl(pi * m / c.N));
-                twf[2 * i] = (float)cosl(2.0L * pi * i / c.N);
-                twf[2 * i + 1] = (float)(-sinl(2.0L * pi * i / c.N));
             }
             cudaMemcpy(c.ktab, ktf.data(), sizeof(float) * c.N, cudaMemcpyHostToDevice);
-            cudaMemcpy(c.tw, twf.data(), sizeof(float) * 2 * c.N, cudaMemcpyHostToDevice);
         } else {
             cudaMemcpy(c.ktab, kt.data(), sizeof(double) * c.N, cudaMemcpyHostToDevice);
-            cudaMemcpy(c.tw, tw.data(), sizeof(double) * 2 * c.N, cudaMemcpyHostToDevice);
         }
     }
     cudaMemset(c.dscal, 0, sizeof(double) * (8 + 1024));
@@ -804,7 +791,7 @@ void pm_destroy(pm_ctx *ctx)
     if (c.stream) cudaStreamSynchronize(c.stream);
     else cudaDeviceSynchronize();
     void *ps[] = {c.part[0], c.part[1], c.count, c.start, c.blocksum, c.phi[0], c.phi[1], c.phi[2], c.chi, c.B,
-                  c.src, c.spec, c.tens, c.ktab, c.tw, c.tw2, c.dscal, c.stage_buf, c.bstate};
+                  c.src, c.spec, c.tens, c.ktab, c.tw2, c.dscal, c.stage_buf, c.bstate};
     for (void *p : ps)
         if (p) cudaFree(p);
     for (auto &row : c.evr)

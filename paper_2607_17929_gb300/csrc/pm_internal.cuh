@@ -68,14 +68,6 @@ struct StepScalars {
     double b_decay;      // (a_{n-1} / a_n)^2
 };
 
-struct FftPlan {
-    int n;
-    int nst;
-    int radix[12];
-};
-
-FftPlan make_plan(int n);
-
 // ---------------------------------------------------------------------------
 // Context.
 // ---------------------------------------------------------------------------
@@ -121,13 +113,11 @@ struct Ctx {
     void *corr = nullptr;       // force correction FP32 [cell][8] (channels 0..2) kicked in by pm_update; not owned
     float corr_scale = 1.f;     // force units per unit of corr
     void *ktab = nullptr;       // N values of ktilde(n)
-    void *tw = nullptr;         // N twiddles exp(-2 pi i k / N)
-    void *tw2 = nullptr;        // per-stage twiddles of the compile-time-N passes
+    void *tw2 = nullptr;        // per-stage twiddles of the FFT passes
     double *dscal = nullptr;    // device f64 scalars: [0] k=0 particle sum, [1..3] mean phi per ring slot,
                                 // [4] (int) record check of a load, [5] (int) latched check of the async puts
     void *stage_buf = nullptr;  // host-transfer staging (f64)
     int64_t stage_elems = 0;
-    FftPlan plan;
 
     // per-kernel CUDA events of the last RING steps (timing window) and the
     // number of library kernels launched
@@ -230,8 +220,7 @@ template <class T>
 pm_status do_solve(Ctx &c, bool bootstrap);   // forward FFTs, Fourier solve, inverse FFTs
 void rotate(Ctx &c);                          // the phi ring after a completed step
 
-// compile-time-N FFT passes (pm_fft.cu)
-bool fast_fft_supported(int n);
+// FFT passes (pm_fft.cu)
 // column-pass shapes: force_* >= 0 selects one, < 0 times the choices and keeps the fastest;
 // false (shape 0 kept) when the context's precision and N have no choice
 template <class T>

@@ -25,9 +25,8 @@ constexpr size_t na_round(size_t b) { return (b + 255) / 256 * 256; }
 constexpr size_t NA_RHO = na_round(sizeof(double) * NA_MAX_MESH * NA_MAX_MESH * NA_MAX_MESH);
 constexpr size_t NA_SPEC = na_round(sizeof(double2) * NA_MAX_MESH * NA_MAX_MESH * (NA_MAX_MESH / 2 + 1));
 constexpr size_t NA_ACC = na_round(sizeof(double) * 3 * NA_MAX_BINS);
-constexpr size_t NA_TW = na_round(sizeof(double2) * NA_MAX_MESH);
 constexpr size_t NA_TW2 = na_round(sizeof(double2) * (2 * NA_MAX_MESH + 64));
-constexpr size_t NA_BYTES = NA_RHO + NA_SPEC + NA_ACC + NA_TW + NA_TW2;
+constexpr size_t NA_BYTES = NA_RHO + NA_SPEC + NA_ACC + NA_TW2;
 
 // The scratch.  In host code this name is only a stand-in for the symbol:
 // the device address comes from cudaGetSymbolAddress (once per device).
@@ -37,14 +36,9 @@ constexpr int NA_MAX_DEVICES = 64;
 std::mutex g_na_mutex;
 void *g_na_addr[NA_MAX_DEVICES] = {};
 
-// twiddles exp(-2 pi i k/n) and the per-stage tables of the compile-time-N passes
-__global__ void k_na_twiddles(int n, double2 *tw, double2 *tw2)
+// the per-stage twiddle tables of the FFT passes
+__global__ void k_na_twiddles(int n, double2 *tw2)
 {
-    for (int k = threadIdx.x; k < n; k += blockDim.x) {
-        double s, c;
-        sincospi(-2.0 * (double)k / (double)n, &s, &c);
-        tw[k] = make_double2(c, s);
-    }
     const int ns = fftc::nstages(n);
     for (int st = 1; st < ns; st++) {
         const int Ns = fftc::span_before(n, st), R = fftc::radix_at(n, st), off = fftc::tw_offset(n, st);
@@ -144,8 +138,7 @@ extern "C" pm_status pm_power_spectrum_noalloc(const double *d_pos, int64_t n_pa
     double *rho = reinterpret_cast<double *>(b);
     double2 *spec = reinterpret_cast<double2 *>(b + NA_RHO);
     double *acc = reinterpret_cast<double *>(b + NA_RHO + NA_SPEC);
-    double2 *tw = reinterpret_cast<double2 *>(b + NA_RHO + NA_SPEC + NA_ACC);
-    double2 *tw2 = reinterpret_cast<double2 *>(b + NA_RHO + NA_SPEC + NA_ACC + NA_TW);
+    double2 *tw2 = reinterpret_cast<double2 *>(b + NA_RHO + NA_SPEC + NA_ACC);
 
     // a context shell pointing at the scratch: no allocation, no timing
     Ctx c;
@@ -155,11 +148,9 @@ extern "C" pm_status pm_power_spectrum_noalloc(const double *d_pos, int64_t n_pa
     c.nc = (int64_t)n_mesh * n_mesh * n_mesh;
     c.nh = (int64_t)n_mesh * n_mesh * (n_mesh / 2 + 1);
     c.np = n_part;
-    c.tw = tw;
     c.tw2 = tw2;
-    c.plan = make_plan(n_mesh);
 
-    k_na_twiddles<<<1, 256, 0, c.stream>>>(n_mesh, tw, tw2);
+    k_na_twiddles<<<1, 256, 0, c.stream>>>(n_mesh, tw2);
     cudaMemsetAsync(rho, 0, sizeof(double) * c.nc, c.stream);
     const double q = (double)c.nc / (double)n_part;  // N^3 m / omega_m with m = omega_m / n_part
     k_na_density<<<(unsigned)((n_part + 255) / 256), 256, 0, c.stream>>>(d_pos, n_part, n_mesh, q, rho);
