@@ -435,8 +435,7 @@ template <class T> pm_status power_t(Ctx &c, int nbins, double *k, double *pk, i
     fft_forward<T>(c, 1, sr, sp);
     CKL("fft");
     double *acc = reinterpret_cast<double *>(c.stage_buf);
-    CK(cudaMemsetAsync(acc, 0, sizeof(double) * 3 * nbins, c.stream));
-    launch_pk_bin<T>(c, sp[0], nbins, acc);
+    launch_pk_bin<T>(c, sp[0], nbins, acc, reinterpret_cast<unsigned int *>(sp[1]));   // sp[1] holds nothing now
     CKL("pk_bin");
     std::vector<double> h(3 * nbins);
     CK(cudaMemcpyAsync(h.data(), acc, sizeof(double) * 3 * nbins, cudaMemcpyDeviceToHost, c.stream));

@@ -153,6 +153,18 @@ struct Ctx {
 enum { EV_START = 0, EV_PROJECT = 1, EV_FWD_X = 2, EV_FWD_Y = 3, EV_FWD_Z = 4, EV_SOLVE = 5,
        EV_INV_Z = 6, EV_INV_Y = 7, EV_INV_X = 8, EV_KICK = 9, EV_SCAN = 10, EV_END = 11 };
 
+// FP32 to FP64 on the integer pipes (the conversion instruction runs on the FP64 pipe); the common range inline
+static __device__ __noinline__ double f32_to_f64_any(float f) { return (double)f; }
+static __device__ __forceinline__ double f32_to_f64(float f)
+{
+    const uint32_t b = __float_as_uint(f), e = (b >> 23) & 255;
+    if (e - 1u < 254u)   // normal
+        return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
+    return (b << 1) == 0 ? __hiloint2double((int)b, 0) : f32_to_f64_any(f);
+}
+static __device__ __forceinline__ double widen(float f) { return f32_to_f64(f); }
+static __device__ __forceinline__ double widen(double f) { return f; }
+
 // True the first time it is called with `mask` on the current device (for per-device one-time set-up
 // such as kernel attributes; a repeated set-up from a racing thread is harmless).
 inline bool first_on_device(std::atomic<uint64_t> &mask)
@@ -203,8 +215,10 @@ void launch_put_packed_sorted(Ctx &c, const pm_packed_particle *in, int *d_bad);
 void launch_store_packed(Ctx &c, pm_packed_particle *out, int64_t first, int64_t count);
 template <class T>
 void launch_density(Ctx &c, void *real_out);
+// P(k) sums of one half spectrum into d_acc [3][nbins]; hist: scratch of pk_hist_len(N) words
+inline int64_t pk_hist_len(int n) { return 3 * (int64_t)(n / 2) * (n / 2) + 1; }
 template <class T>
-void launch_pk_bin(Ctx &c, const void *spec_in, int nbins, double *d_acc);
+void launch_pk_bin(Ctx &c, const void *spec_in, int nbins, double *d_acc, unsigned int *hist);
 template <class T>
 void launch_to_f64(Ctx &c, const void *src, double *dst, int64_t n);
 template <class T>

@@ -26,7 +26,8 @@ constexpr size_t NA_RHO = na_round(sizeof(double) * NA_MAX_MESH * NA_MAX_MESH * 
 constexpr size_t NA_SPEC = na_round(sizeof(double2) * NA_MAX_MESH * NA_MAX_MESH * (NA_MAX_MESH / 2 + 1));
 constexpr size_t NA_ACC = na_round(sizeof(double) * 3 * NA_MAX_BINS);
 constexpr size_t NA_TW2 = na_round(sizeof(double2) * (2 * NA_MAX_MESH + 64));
-constexpr size_t NA_BYTES = NA_RHO + NA_SPEC + NA_ACC + NA_TW2;
+constexpr size_t NA_HIST = na_round(sizeof(unsigned int) * (3 * (NA_MAX_MESH / 2) * (NA_MAX_MESH / 2) + 1));
+constexpr size_t NA_BYTES = NA_RHO + NA_SPEC + NA_ACC + NA_TW2 + NA_HIST;
 
 // The scratch.  In host code this name is only a stand-in for the symbol:
 // the device address comes from cudaGetSymbolAddress (once per device).
@@ -139,6 +140,7 @@ extern "C" pm_status pm_power_spectrum_noalloc(const double *d_pos, int64_t n_pa
     double2 *spec = reinterpret_cast<double2 *>(b + NA_RHO);
     double *acc = reinterpret_cast<double *>(b + NA_RHO + NA_SPEC);
     double2 *tw2 = reinterpret_cast<double2 *>(b + NA_RHO + NA_SPEC + NA_ACC);
+    unsigned int *hist = reinterpret_cast<unsigned int *>(b + NA_RHO + NA_SPEC + NA_ACC + NA_TW2);
 
     // a context shell pointing at the scratch: no allocation, no timing
     Ctx c;
@@ -158,8 +160,7 @@ extern "C" pm_status pm_power_spectrum_noalloc(const double *d_pos, int64_t n_pa
     const void *in[1] = {rho};
     void *out[1] = {spec};
     fft_forward<double>(c, 1, in, out);
-    cudaMemsetAsync(acc, 0, sizeof(double) * 3 * nbins, c.stream);
-    launch_pk_bin<double>(c, spec, nbins, acc);
+    launch_pk_bin<double>(c, spec, nbins, acc, hist);
     double h[3 * NA_MAX_BINS];
     cudaError_t e = cudaMemcpyAsync(h, acc, sizeof(double) * 3 * nbins, cudaMemcpyDeviceToHost, c.stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c.stream);

@@ -56,6 +56,13 @@ template <> struct Acc<float> {
         s = __fadd_rn(s, h);
         c = __fadd_rn(c, __fsub_rn(x, h));
     }
+    // += x + lo
+    __device__ __forceinline__ void add_split(float x, float lo, float M)
+    {
+        const float h = __fsub_rn(__fadd_rn(x, M), M);
+        s = __fadd_rn(s, h);
+        c = __fadd_rn(c, __fadd_rn(__fsub_rn(x, h), lo));
+    }
     __device__ __forceinline__ float hi() const { return s; }
     __device__ __forceinline__ float lo() const { return c; }
 };
@@ -275,14 +282,14 @@ constexpr int NDEPSHAPES = 2;
 
 // sums exchanged per vertex: T00 (two words in FP32) and the other 8 charges
 template <class T, bool FULL> constexpr int dep_words() { return (sizeof(T) == 4 ? 2 : 1) + (FULL ? 8 : 0); }
-// words of a particle's weights and charges
-template <bool FULL> constexpr int dep_rec() { return FULL ? 17 : 9; }
+// words of a particle's weights and charges; DEN: its weights in two words instead of charges
+template <bool FULL, bool DEN> constexpr int dep_rec() { return FULL || DEN ? 17 : 9; }
 // staged particle records (the first 32 of a row, two planes), exchange rows (two planes), weights and charges,
 // staged potentials
-template <class T, bool FULL> constexpr size_t dep_smem()
+template <class T, bool FULL, bool DEN> constexpr size_t dep_smem()
 {
     return 2 * DEP_THREADS * sizeof(Particle<T>) +
-           sizeof(T) * 32 * DROWS * (2 * dep_words<T, FULL>() + dep_rec<FULL>()) + sizeof(T) * (FULL ? 2 * DRING * DPN : 0);
+           sizeof(T) * 32 * DROWS * (2 * dep_words<T, FULL>() + dep_rec<FULL, DEN>()) + sizeof(T) * (FULL ? 2 * DRING * DPN : 0);
 }
 
 // (hi, lo) += (h, l) of another sum, TwoSum on the high words
@@ -306,6 +313,24 @@ __device__ __forceinline__ PartFU<double> unpack(const double2 *q, int step)
 {
     const double2 a = q[0], b = q[step], c = q[2 * step], d = q[3 * step];
     return {__double2loint(a.x), {a.y, b.x, b.y}, {c.x, c.y, d.x}};
+}
+
+// The FP32 weights of charges() with the low words that make them exact to 2^-48 (w above its rounding).
+__device__ __forceinline__ void weights_lo(const PartFU<float> &P, const float (&w)[8], float (&lo)[8])
+{
+    float g[3], ge[3];   // 1 - f in two words
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+        g[d] = 1.f - P.f[d];
+        ge[d] = __fsub_rn(__fsub_rn(1.f, g[d]), P.f[d]);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        const float a = i & 1 ? P.f[1] : g[1], ae = i & 1 ? 0.f : ge[1], b = i & 2 ? P.f[2] : g[2], be = i & 2 ? 0.f : ge[2];
+        const float p = __fmul_rn(a, b), e = __fmaf_rn(a, b, -p) + (a * be + ae * b);
+        lo[i] = __fmaf_rn(g[0], p, -w[i]) + (g[0] * e + ge[0] * p);
+        lo[4 + i] = __fmaf_rn(P.f[0], p, -w[4 + i]) + P.f[0] * e;
+    }
 }
 
 // Charges of one particle and its 8 CIC weights (w[4 dx + dy + 2 dz]).  lo/up: the staged potentials of the
@@ -466,10 +491,10 @@ struct DepRow {
 };
 
 // A thread's view of its tile.
-template <class T, bool FULL> struct DepCol {
+template <class T, bool FULL, bool DEN> struct DepCol {
     static constexpr int PQ = sizeof(Particle<T>) / 16;    // 16-byte parts of a record
     static constexpr int VT = 16 / sizeof(T);              // values in 16 bytes
-    static constexpr int W = dep_words<T, FULL>(), R = dep_rec<FULL>();
+    static constexpr int W = dep_words<T, FULL>(), R = dep_rec<FULL, DEN>();
     using V = std::conditional_t<sizeof(T) == 4, float4, double2>;
 
     const DepParams<T> &p;
@@ -573,6 +598,12 @@ template <class T, bool FULL> struct DepCol {
 #pragma unroll
                 for (int k = 0; k < 8 / VT; k++) rv[32 * (8 / VT + k) + lane] = pack(q + VT * k);
             }
+            if constexpr (DEN) {
+                float wlo[8];
+                weights_lo(P, wt, wlo);
+#pragma unroll
+                for (int k = 0; k < 2; k++) rv[32 * (2 + k) + lane] = pack(wlo + 4 * k);
+            }
             T *r0 = rec + 32 * (R - 1);
             r0[lane] = q00;
             __syncwarp();
@@ -584,6 +615,14 @@ template <class T, bool FULL> struct DepCol {
                     const V *v = rv + n + (n < nm ? 32 * (4 / VT) : 0);
 #pragma unroll
                     for (int k = 0; k < 4 / VT; k++) unpackv(v[32 * k], wn + VT * k);
+                    if constexpr (DEN) {
+                        unpackv(v[64], qn);
+                        A.t00[0].add_split(wn[0], qn[0], p.magic);
+                        A.t00[1].add_split(wn[1], qn[1], p.magic);
+                        B.t00[0].add_split(wn[2], qn[2], p.magic);
+                        B.t00[1].add_split(wn[3], qn[3], p.magic);
+                        continue;
+                    }
                     const T t = r0[n];
                     A.t00[0].add_product(wn[0], t, p.magic);
                     A.t00[1].add_product(wn[1], t, p.magic);
@@ -627,7 +666,12 @@ template <class T, bool FULL> struct DepCol {
             T dS = (A.t00[0].hi() + xi[0]) - p.rb_hi;
             if constexpr (sizeof(T) == 4) dS += (A.t00[0].lo() + xi[32]) - p.rb_lo;
             const int g = cells + lane;
-            if constexpr (!FULL) {
+            if constexpr (DEN) {
+                // the contrast N^3 / n_part (S - n_part / N^3) in two words
+                const float h = (A.t00[0].hi() + xi[0]) - p.rb_hi, l = (A.t00[0].lo() + xi[32]) - p.rb_lo;
+                const float sum = __fadd_rn(h, l), low = __fsub_rn(l, __fsub_rn(sum, h)), x = __fmul_rn(p.G, sum);
+                reinterpret_cast<T *>(p.out.p[0])[g] = x + (__fmaf_rn(p.G, sum, -x) + (p.G * low + p.c1 * sum));
+            } else if constexpr (!FULL) {
                 reinterpret_cast<T *>(p.out.p[0])[g] = p.G * dS;
             } else {
                 T s[8];
@@ -642,12 +686,12 @@ template <class T, bool FULL> struct DepCol {
 };
 
 // The deposit of tile b of the box described by p.
-template <class T, bool FULL>
+template <class T, bool FULL, bool DEN = false>
 __device__ __forceinline__ void deposit_tile(const DepParams<T> &p, const int b)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const int N = p.N, tid = threadIdx.x, w = tid >> 5;
-    using C = DepCol<T, FULL>;
+    using C = DepCol<T, FULL, DEN>;
     C c{p};
     c.stage = reinterpret_cast<typename C::V *>(smem);
     c.rec = reinterpret_cast<T *>(smem + 2 * DEP_THREADS * sizeof(Particle<T>)) + w * (32 * C::R);
@@ -701,6 +745,14 @@ template <class T, bool FULL>
 __global__ void __launch_bounds__(DEP_THREADS, dep_ctas<T, FULL>()) k_project(const __grid_constant__ DepParams<T> p)
 {
     deposit_tile<T, FULL>(p, blockIdx.x);
+}
+
+// The CIC density contrast of the P(k) diagnostic in FP32 contexts: the columns above with the weights and the sums
+// in two words.  In place of FP64 weights and atomics on the FP64 pipe: 256^3 0.98 (with clearing and the final
+// pass) -> 0.26 ms; FP64 contexts take k_project with unit mass, 1.0 -> 0.5.
+__global__ void __launch_bounds__(DEP_THREADS, 2) k_contrast(const __grid_constant__ DepParams<float> p)
+{
+    deposit_tile<float, false, true>(p, blockIdx.x);
 }
 
 // Several boxes in one launch (the batched ensemble): CTA j deposits tile j - first[i] of box i, the box whose
@@ -1214,7 +1266,6 @@ __global__ void __launch_bounds__(256) k_scatter(const Particle<T> *in, Particle
 // the compiler would otherwise run both and select.
 // ---------------------------------------------------------------------------
 __device__ __noinline__ float f64_to_f32_any(double d) { return (float)d; }
-__device__ __noinline__ double f32_to_f64_any(float f) { return (double)f; }
 __device__ __noinline__ double position_any(int c, float f, double inv_n) { return ((double)c + (double)f) * inv_n; }
 __device__ __noinline__ double wrap_unit(double x)
 {
@@ -1231,14 +1282,6 @@ __device__ __forceinline__ float f64_to_f32(double d)
         return __uint_as_float(sign | ((uint32_t)((m + 0x0fffffffull + ((m >> 29) & 1)) >> 29) - (896u << 23)));
     return e == 0 ? __uint_as_float(sign) : f64_to_f32_any(d);
 }
-__device__ __forceinline__ double f32_to_f64(float f)
-{
-    const uint32_t b = __float_as_uint(f), e = (b >> 23) & 255;
-    if (e - 1u < 254u)   // normal
-        return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
-    return (b << 1) == 0 ? __hiloint2double((int)b, 0) : f32_to_f64_any(f);
-}
-
 // Integer part (returned) and fraction of s in [0, 2^10].
 __device__ __forceinline__ int split(double s, double &f)
 {
@@ -1293,11 +1336,9 @@ __device__ __forceinline__ double position(int c, float f, double inv_n, double 
     return position_any(c, f, inv_n);
 }
 
-// the two conversions above where the particle type is f32
+// f64_to_f32 where the particle type is f32
 __device__ __forceinline__ void narrow(double d, float &f) { f = f64_to_f32(d); }
 __device__ __forceinline__ void narrow(double d, double &f) { f = d; }
-__device__ __forceinline__ double widen(float f) { return f32_to_f64(f); }
-__device__ __forceinline__ double widen(double f) { return f; }
 
 // ---------------------------------------------------------------------------
 // Particle I/O: f64 (x, y, z) rows <-> cell + offset records.
@@ -1490,34 +1531,6 @@ __global__ void __launch_bounds__(256) k_store(const Particle<T> *byid, int64_t 
     }
 }
 
-// CIC mass density contrast delta = rho/omega_m - 1 (diagnostic, global FP64 atomics).
-template <class T>
-__global__ void k_density_acc(const Particle<T> *part, int64_t np, int N, double q, double *rho)
-{
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= np) return;
-    const Particle<T> P = part[i];
-    const int ix = P.cell % N, iy = (P.cell / N) % N, iz = P.cell / (N * N);
-    const double f[3] = {(double)P.f[0], (double)P.f[1], (double)P.f[2]};
-#pragma unroll
-    for (int dz = 0; dz < 2; dz++)
-#pragma unroll
-        for (int dy = 0; dy < 2; dy++)
-#pragma unroll
-            for (int dx = 0; dx < 2; dx++) {
-                const double w = (dx ? f[0] : 1 - f[0]) * (dy ? f[1] : 1 - f[1]) * (dz ? f[2] : 1 - f[2]);
-                const int64_t g = ((int64_t)wrapi(iz + dz, N) * N + wrapi(iy + dy, N)) * N + wrapi(ix + dx, N);
-                atomicAdd(&rho[g], q * w);
-            }
-}
-
-template <class T>
-__global__ void k_density_fin(const double *rho, int64_t n, T *out)
-{
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = (T)(rho[i] - 1.0);
-}
-
 template <class T> __global__ void k_to_f64(const T *s, double *d, int64_t n)
 {
     // four values a thread: with one, starting the blocks takes longer than the copy
@@ -1620,10 +1633,10 @@ template <class T, bool FULL> void dep_attrs()
 {
     static std::atomic<uint64_t> attr{0};
     if (first_on_device(attr)) {
-        cudaFuncSetAttribute(k_project<T, FULL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dep_smem<T, FULL>());
+        cudaFuncSetAttribute(k_project<T, FULL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dep_smem<T, FULL, false>());
         if constexpr (sizeof(T) == 8 || FULL)
             cudaFuncSetAttribute(k_project_batch<T, FULL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)dep_smem<T, FULL>());
+                                 (int)dep_smem<T, FULL, false>());
     }
 }
 
@@ -1641,10 +1654,10 @@ void launch_project(Ctx &c, const StepScalars &s)
     cudaMemsetAsync(c.dscal + 8, 0, sizeof(double) * NK0SLOTS, c.stream);
     if (dep_full(s)) {
         dep_attrs<T, true>();
-        k_project<T, true><<<dep_ntiles(p), DEP_THREADS, dep_smem<T, true>(), c.stream>>>(p);
+        k_project<T, true><<<dep_ntiles(p), DEP_THREADS, dep_smem<T, true, false>(), c.stream>>>(p);
     } else if (!dep_mass(p)) {
         dep_attrs<T, false>();
-        k_project<T, false><<<dep_ntiles(p), DEP_THREADS, dep_smem<T, false>(), c.stream>>>(p);
+        k_project<T, false><<<dep_ntiles(p), DEP_THREADS, dep_smem<T, false, false>(), c.stream>>>(p);
     } else if constexpr (sizeof(T) == 4) {
         k_mass<<<dep_ntiles(p), MTHREADS, 0, c.stream>>>(p);
     }
@@ -1672,12 +1685,12 @@ void launch_project_batch(Ctx *const *cs, const StepScalars *ss, int n, bool ful
         }
         if (full) {
             dep_attrs<T, true>();
-            k_project_batch<T, true><<<q.first[nb], DEP_THREADS, dep_smem<T, true>(), st>>>(q);
+            k_project_batch<T, true><<<q.first[nb], DEP_THREADS, dep_smem<T, true, false>(), st>>>(q);
         } else if constexpr (sizeof(T) == 4) {
             k_mass_batch<<<q.first[nb], MTHREADS, 0, st>>>(q);
         } else {
             dep_attrs<T, false>();
-            k_project_batch<T, false><<<q.first[nb], DEP_THREADS, dep_smem<T, false>(), st>>>(q);
+            k_project_batch<T, false><<<q.first[nb], DEP_THREADS, dep_smem<T, false, false>(), st>>>(q);
         }
         k_k0_reduce_batch<<<nb, 1024, 0, st>>>(kq);
     }
@@ -1882,15 +1895,34 @@ void launch_store_packed(Ctx &c, pm_packed_particle *out, int64_t first, int64_t
         reinterpret_cast<const Particle<float> *>(c.part[1 - c.cur]), first, count, out, vec);
 }
 
+// CIC mass density contrast delta = rho / omega_m - 1
 template <class T>
 void launch_density(Ctx &c, void *real_out)
 {
-    double *rho = reinterpret_cast<double *>(c.spec);  // scratch: nc doubles fit in the spectra block
-    cudaMemsetAsync(rho, 0, sizeof(double) * c.nc, c.stream);
-    const double q = (double)c.nc / (double)c.np;  // N^3 m / omega_m
-    k_density_acc<T><<<nblk(c.np, 256), 256, 0, c.stream>>>(reinterpret_cast<const Particle<T> *>(c.part[c.cur]),
-                                                             c.np, c.N, q, rho);
-    k_density_fin<T><<<nblk(c.nc, 256), 256, 0, c.stream>>>(rho, c.nc, reinterpret_cast<T *>(real_out));
+    DepParams<T> p{};
+    p.part = reinterpret_cast<const Particle<T> *>(c.part[c.cur]);
+    p.start = c.start;
+    p.out.p[0] = real_out;
+    p.N = c.N;
+    p.newtonian = 1;
+    p.mass = T(1);
+    dep_tiles(p, false, c.dep_shape);
+    const double mean = (double)c.np / (double)c.nc, q = (double)c.nc / (double)c.np;
+    p.G = (T)q;
+    p.c1 = (T)(q - (double)p.G);
+    p.rb_hi = (T)mean;
+    p.rb_lo = (T)(mean - (double)p.rb_hi);
+    p.magic = (T)std::ldexp(1.5, std::ilogb(std::max(1.0, mean)) + 1 - 13 + 23);
+    const int nt = p.ntx * p.nty * ((p.N + p.tz - 1) / p.tz);
+    if constexpr (sizeof(T) == 4) {
+        static std::atomic<uint64_t> attr{0};
+        constexpr int bytes = (int)dep_smem<float, false, true>();
+        if (first_on_device(attr)) cudaFuncSetAttribute(k_contrast, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        k_contrast<<<nt, DEP_THREADS, bytes, c.stream>>>(p);
+    } else {
+        dep_attrs<T, false>();
+        k_project<T, false><<<nt, DEP_THREADS, dep_smem<T, false, false>(), c.stream>>>(p);
+    }
 }
 
 template <class T>
