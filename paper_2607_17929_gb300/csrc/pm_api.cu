@@ -218,7 +218,7 @@ template <class T> pm_status do_solve(Ctx &c, bool bootstrap)
                      reinterpret_cast<T *>(c.B) + 2 * c.nc, c.chi};
     fft_inverse<T>(c, full ? 5 : 1, sp, outs);
     CKL("fft_inverse");
-    if (!full) {
+    if (bootstrap) {   // the Newtonian mode never writes them, so they stay as its bootstrap leaves them
         CK(cudaMemsetAsync(c.chi, 0, sizeof(T) * c.nc, c.stream));
         CK(cudaMemsetAsync(c.B, 0, sizeof(T) * 3 * c.nc, c.stream));
     }
@@ -322,7 +322,7 @@ pm_status set_particles_t(Ctx &c, const double *pos, const double *mom, bool boo
     CK(cudaMemsetAsync(c.chi, 0, sizeof(T) * c.nc, c.stream));
     CK(cudaMemsetAsync(c.tens, 0, sizeof(typename Cplx<T>::type) * 4 * c.nh, c.stream));
     if (c.bstate) CK(cudaMemsetAsync(c.bstate, 0, sizeof(typename Cplx<T>::type) * 3 * c.nh, c.stream));
-    CK(cudaMemsetAsync(c.dscal, 0, sizeof(double) * 8, c.stream));
+    CK(cudaMemsetAsync(c.dscal, 0, sizeof(double) * (8 + NK0SLOTS), c.stream));
     c.step = 0;
     pm_status st = do_project<T>(c, true);
     if (st) return st;
@@ -574,6 +574,7 @@ template <class T> pm_status load_impl(Ctx &c, const char *path)
     CK(cudaStreamSynchronize(c.stream));
     // the cell index (count / start) is rebuilt by the caller (recount)
     CK(cudaMemsetAsync(c.count, 0, sizeof(int32_t) * c.nc, c.stream));
+    CK(cudaMemsetAsync(c.dscal + 8, 0, sizeof(double) * NK0SLOTS, c.stream));   // of a projection without its solve
     c.step = h.step;
     c.stage = 0;
     c.have_particles = true;
@@ -718,7 +719,7 @@ pm_status pm_init(const pm_config *cfg, pm_ctx **out)
         {&c.tens, 4 * 2 * ts * (size_t)c.nh},
         {&c.ktab, ts * (size_t)c.N},
         {&c.tw2, 2 * ts * (size_t)(2 * c.N + 64)},
-        {(void **)&c.dscal, sizeof(double) * (8 + 1024)},
+        {(void **)&c.dscal, sizeof(double) * (8 + NK0SLOTS)},
         {&c.stage_buf, sizeof(double) * (size_t)c.stage_elems},
         {&c.bstate, c.b_space ? 3 * 2 * ts * (size_t)c.nh : 0},   // 0: not needed
     };
@@ -762,7 +763,7 @@ pm_status pm_init(const pm_config *cfg, pm_ctx **out)
             cudaMemcpy(c.ktab, kt.data(), sizeof(double) * c.N, cudaMemcpyHostToDevice);
         }
     }
-    cudaMemset(c.dscal, 0, sizeof(double) * (8 + 1024));
+    cudaMemset(c.dscal, 0, sizeof(double) * (8 + NK0SLOTS));
     cudaMemset(c.phi[0], 0, ts * c.nc);
     cudaMemset(c.phi[1], 0, ts * c.nc);
     cudaMemset(c.phi[2], 0, ts * c.nc);

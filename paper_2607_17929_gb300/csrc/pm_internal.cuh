@@ -40,6 +40,9 @@ template <> struct alignas(16) Particle<double> {
 static_assert(sizeof(Particle<float>) == 32, "mixed particle must be 32 B");
 static_assert(sizeof(Particle<double>) == 64, "fp64 particle must be 64 B");
 
+// slots of partial sums of the k = 0 excess (dscal[8] ..): the projection adds to them, the solve sums and clears them
+constexpr int NK0SLOTS = 1024;
+
 // Up to 16 device pointers for batched multi-field launches.
 struct Ptrs {
     void *p[16];
@@ -114,7 +117,7 @@ struct Ctx {
     float corr_scale = 1.f;     // force units per unit of corr
     void *ktab = nullptr;       // N values of ktilde(n)
     void *tw2 = nullptr;        // per-stage twiddles of the FFT passes
-    double *dscal = nullptr;    // device f64 scalars: [0] k=0 particle sum, [1..3] mean phi per ring slot,
+    double *dscal = nullptr;    // device f64 scalars: [1..3] mean phi per ring slot, [8..] the k = 0 slots,
                                 // [4] (int) record check of a load, [5] (int) latched check of the async puts
     void *stage_buf = nullptr;  // host-transfer staging (f64)
     int64_t stage_elems = 0;

@@ -20,7 +20,6 @@ namespace pm {
 
 namespace {
 
-constexpr int NK0SLOTS = 1024;
 
 // Per-cell accumulator of the T^00 charge, whose cell sums cancel against the
 // uniform background in R.  FP64: plain double.  Mixed: float-float with
@@ -162,6 +161,7 @@ __device__ __forceinline__ T hc_remainder(T ph, const T (&up)[3], const T (&dn)[
 // records and searched each particle's cell.
 // ---------------------------------------------------------------------------
 constexpr int MT = 8, MR = MT + 1, MCELLS = MR * MR * MR, MTHREADS = MT * MT * MT;
+constexpr int MOWN = 8;     // particles of two cells that their thread stages itself
 constexpr int MCAP = 960;   // particles staged at a time (a nearly uniform load of one per cell has 729)
 
 struct MassSmem {
@@ -212,21 +212,22 @@ __device__ __forceinline__ void mass_tile(const DepParams<float> &p, const int b
     acc.zero();
     for (int lo = 0; lo < total; lo += MCAP) {
         const int hi = min(total, lo + MCAP);
-        // each thread stages the particles of its two cells, two loads under way at a time
-        const int last = n[0] + n[1];
-        for (int k = max(lo - e, 0); k < min(last, hi - e); k += 2) {
-            float2 xy[2];
-            float z[2];
-#pragma unroll
-            for (int j = 0; j < 2; j++)
-                if (k + j < last) {
-                    const float *q = reinterpret_cast<const float *>(p.part + (k + j < n[0] ? s[0] + k + j : s[1] + (k + j - n[0])));
-                    xy[j] = __ldg(reinterpret_cast<const float2 *>(q + 2));
-                    z[j] = __ldg(q + 4);
-                }
-#pragma unroll
-            for (int j = 0; j < 2; j++)
-                if (k + j < last && e + k + j < hi) sm.rec[e + k + j - lo] = make_float4(xy[j].x, xy[j].y, z[j], 0.f);
+        // each thread stages the particles of its two cells, MOWN at most; the warp
+        // together stages what is left in crowded cells
+        auto stage = [&](int first0, int n0, int first1, int k, int to) {
+            const float *q = reinterpret_cast<const float *>(p.part + (k < n0 ? first0 + k : first1 + (k - n0)));
+            const float2 xy = __ldg(reinterpret_cast<const float2 *>(q + 2));
+            sm.rec[to] = make_float4(xy.x, xy.y, __ldg(q + 4), 0.f);
+        };
+        const int k0 = max(lo - e, 0), k1 = min(n[0] + n[1], hi - e), ko = min(k1, k0 + MOWN);
+#pragma unroll 1
+        for (int k = k0; k < ko; k++) stage(s[0], n[0], s[1], k, e + k - lo);
+        for (unsigned left = __ballot_sync(0xffffffffu, ko < k1); left; left &= left - 1) {
+            const int o = __ffs(left) - 1;
+            const int f0 = __shfl_sync(0xffffffffu, s[0], o), m0 = __shfl_sync(0xffffffffu, n[0], o),
+                      f1 = __shfl_sync(0xffffffffu, s[1], o), to = __shfl_sync(0xffffffffu, e, o) - lo,
+                      end = __shfl_sync(0xffffffffu, k1, o);
+            for (int k = __shfl_sync(0xffffffffu, ko, o) + lane; k < end; k += 32) stage(f0, m0, f1, k, to + k);
         }
         __syncthreads();
         // vertex o receives from cells o - d, d in {0,1}^3, weight (d ? f : 1 - f) per axis; the x-neighbours
@@ -778,30 +779,6 @@ __global__ void __launch_bounds__(MTHREADS, 4) k_mass_batch(const __grid_constan
     int i = 0;
     while (i + 1 < q.nbox && (int)blockIdx.x >= q.first[i + 1]) i++;
     mass_tile(q.box[i], (int)blockIdx.x - q.first[i]);
-}
-
-// Sum the k = 0 slots: dscal[0] = sum over particles of the T^00 excess (block b: box b of a batch).
-struct K0Batch {
-    double *dscal[MAXBATCH];
-};
-__device__ void k0_reduce_one(double *dscal);
-__global__ void k_k0_reduce(double *dscal) { k0_reduce_one(dscal); }
-__global__ void k_k0_reduce_batch(const __grid_constant__ K0Batch q) { k0_reduce_one(q.dscal[blockIdx.x]); }
-__device__ void k0_reduce_one(double *dscal)
-{
-    __shared__ double s[32];
-    double v = 0.0;
-    for (int i = threadIdx.x; i < NK0SLOTS; i += blockDim.x) v += dscal[8 + i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        v = threadIdx.x < (blockDim.x >> 5) ? s[threadIdx.x] : 0.0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (threadIdx.x == 0) dscal[0] = v;
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1651,7 +1628,6 @@ template <class T>
 void launch_project(Ctx &c, const StepScalars &s)
 {
     const DepParams<T> p = dep_params<T>(c, s);
-    cudaMemsetAsync(c.dscal + 8, 0, sizeof(double) * NK0SLOTS, c.stream);
     if (dep_full(s)) {
         dep_attrs<T, true>();
         k_project<T, true><<<dep_ntiles(p), DEP_THREADS, dep_smem<T, true, false>(), c.stream>>>(p);
@@ -1661,8 +1637,7 @@ void launch_project(Ctx &c, const StepScalars &s)
     } else if constexpr (sizeof(T) == 4) {
         k_mass<<<dep_ntiles(p), MTHREADS, 0, c.stream>>>(p);
     }
-    k_k0_reduce<<<1, 1024, 0, c.stream>>>(c.dscal);
-    c.launches += 2;
+    c.launches++;
 }
 
 // One deposit launch over several boxes of one precision, all relativistic or all Newtonian (batches of MAXBATCH).
@@ -1672,16 +1647,13 @@ void launch_project_batch(Ctx *const *cs, const StepScalars *ss, int n, bool ful
     for (int b0 = 0; b0 < n; b0 += MAXBATCH) {
         const int nb = std::min(MAXBATCH, n - b0);
         thread_local DepBatch<T> q;   // host staging of the launch parameters (copied at launch)
-        K0Batch kq{};
         q.nbox = nb;
         q.first[0] = 0;
         for (int i = 0; i < nb; i++) {
             Ctx &c = *cs[b0 + i];
             q.box[i] = dep_params<T>(c, ss[b0 + i]);
             q.first[i + 1] = q.first[i] + dep_ntiles(q.box[i]);
-            kq.dscal[i] = c.dscal;
-            cudaMemsetAsync(c.dscal + 8, 0, sizeof(double) * NK0SLOTS, st);
-            c.launches += 2;
+            c.launches++;
         }
         if (full) {
             dep_attrs<T, true>();
@@ -1692,7 +1664,6 @@ void launch_project_batch(Ctx *const *cs, const StepScalars *ss, int n, bool ful
             dep_attrs<T, false>();
             k_project_batch<T, false><<<q.first[nb], DEP_THREADS, dep_smem<T, false, false>(), st>>>(q);
         }
-        k_k0_reduce_batch<<<nb, 1024, 0, st>>>(kq);
     }
 }
 
@@ -1785,8 +1756,8 @@ void launch_kick_batch(Ctx *const *cs, const StepScalars *ss, int n, bool full, 
 
 // Time the deposit of the context's current state with each chunk capacity and keep the fastest.  The trial
 // deposits write into the spectrum buffer, which holds nothing between steps (9 half spectra hold more than
-// 9 real fields), so the sources the caller can read stay as they were; the k = 0 scalar they also write is
-// recomputed by the next projection before the solve reads it.
+// 9 real fields), so the sources the caller can read stay as they were; the k = 0 slots they also add to are
+// cleared again.
 template <class T>
 int tune_deposit_shape(Ctx &c, const StepScalars &s)
 {
@@ -1813,6 +1784,7 @@ int tune_deposit_shape(Ctx &c, const StepScalars &s)
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
+    cudaMemsetAsync(c.dscal + 8, 0, sizeof(double) * NK0SLOTS, c.stream);
     c.src = src;
     c.dep_shape = best_v;
     return best_v;

@@ -25,7 +25,7 @@ template <class T> struct SolveParams {
     void *spec;        // 9 half spectra: R, Fx, Fy, Fz, Sxx, Sxy, Sxz, Syy, Syz
     void *tens;        // 4 half spectra: h+, hx, h+', hx'
     const T *ktab;     // ktilde per DFT index
-    double *dscal;     // [0] particle excess sum, [1 + ring] mean phi per ring slot
+    double *dscal;     // [1 + ring] mean phi per ring slot, [8 ..] slots of the k = 0 excess
     int imean_prev, imean_new;
     int N;
     int64_t nh;
@@ -42,6 +42,24 @@ __global__ void __launch_bounds__(256) k_solve(SolveParams<T> p)
 {
     using C = typename Cplx<T>::type;
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    // the k = 0 excess of the projection: block 0 (whole, as nh >= 320) sums its slots and clears them for the next one
+    double k0 = 0.0;
+    if (blockIdx.x == 0 && !p.newtonian) {
+        __shared__ double part[8];
+        static_assert(NK0SLOTS == 4 * 256, "four slots a thread");
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            k0 += p.dscal[8 + threadIdx.x + 256 * q];
+            p.dscal[8 + threadIdx.x + 256 * q] = 0.0;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) k0 += __shfl_down_sync(0xffffffffu, k0, o);
+        if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = k0;
+        __syncthreads();
+        k0 = 0.0;
+        if (threadIdx.x == 0)
+            for (int q = 0; q < 8; q++) k0 += part[q];
+    }
     if (e >= p.nh) return;
     const int N = p.N, h = N / 2 + 1;
     const int kx = (int)(e % h);
@@ -74,7 +92,7 @@ __global__ void __launch_bounds__(256) k_solve(SolveParams<T> p)
     if (zero) {
         double mean_phi = 0.0;
         if (!p.newtonian) {
-            double mean_r = p.four_pi_g_a2 * p.dscal[0];
+            double mean_r = p.four_pi_g_a2 * k0;
             if (!p.bootstrap) mean_r -= p.c1 * p.dscal[1 + p.imean_prev];
             mean_phi = -mean_r / (p.c1 + p.c2);
         }
