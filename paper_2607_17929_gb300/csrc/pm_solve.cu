@@ -37,6 +37,11 @@ template <class T> struct SolveParams {
     T b_decay, dtau_prev;
 };
 
+// FP64 takes the fewest operations (its pipe bounds the FP64 solve: 256^3 4.5 -> 3.2 ms); FP32, bound by memory, the
+// IEEE square root and quotients.
+__device__ __forceinline__ double inv_sqrt(double x) { return rsqrt(x); }
+__device__ __forceinline__ float inv_sqrt(float x) { return 1.f / sqrtf(x); }
+
 template <class T>
 __global__ void __launch_bounds__(256) k_solve(SolveParams<T> p)
 {
@@ -131,34 +136,53 @@ __global__ void __launch_bounds__(256) k_solve(SolveParams<T> p)
     szz.y = -sxx.y - syy.y;
     const C Sm[3][3] = {{sxx, sxy, sxz}, {sxy, syy, syz}, {sxz, syz, szz}};
 
+    // v_l = kt_i Sig_il and kt_i kt_j Sig_ij
+    C v[3], kks;
+#pragma unroll
+    for (int l = 0; l < 3; l++) {
+        v[l].x = kt[0] * Sm[0][l].x + kt[1] * Sm[1][l].x + kt[2] * Sm[2][l].x;
+        v[l].y = kt[0] * Sm[0][l].y + kt[1] * Sm[1][l].y + kt[2] * Sm[2][l].y;
+    }
+    kks.x = kt[0] * v[0].x + kt[1] * v[1].x + kt[2] * v[2].x;
+    kks.y = kt[0] * v[0].y + kt[1] * v[1].y + kt[2] * v[2].y;
+    const T ik2 = T(1) / k2;
+
     // tensor sector: polarisation basis from the axis with the smallest |n_i|
     {
-        const T kn = sqrt(k2);
-        const T kh[3] = {kt[0] / kn, kt[1] / kn, kt[2] / kn};
+        const T ikn = inv_sqrt(k2);
+        const T kh[3] = {kt[0] * ikn, kt[1] * ikn, kt[2] * ikn};
         int m = 0;
         if (abs(nv[1]) < abs(nv[m])) m = 1;
         if (abs(nv[2]) < abs(nv[m])) m = 2;
-        T e1[3] = {-kh[m] * kh[0], -kh[m] * kh[1], -kh[m] * kh[2]};
-        e1[m] += T(1);
-        const T l = sqrt(e1[0] * e1[0] + e1[1] * e1[1] + e1[2] * e1[2]);
+        const T km = m == 0 ? kh[0] : m == 1 ? kh[1] : kh[2];
+        T e1[3] = {-km * kh[0], -km * kh[1], -km * kh[2]};
 #pragma unroll
-        for (int d = 0; d < 3; d++) e1[d] /= l;
+        for (int d = 0; d < 3; d++) e1[d] += d == m ? T(1) : T(0);
+        const T il = inv_sqrt(e1[0] * e1[0] + e1[1] * e1[1] + e1[2] * e1[2]);
+#pragma unroll
+        for (int d = 0; d < 3; d++) e1[d] *= il;
         const T e2[3] = {kh[1] * e1[2] - kh[2] * e1[1], kh[2] * e1[0] - kh[0] * e1[2],
                          kh[0] * e1[1] - kh[1] * e1[0]};
-        const T is2 = T(0.70710678118654752440084436210484903928);
+        // e^+_ij Sig_ij = (e1 Sig e1 - e2 Sig e2) / sqrt2, e^x_ij Sig_ij = sqrt2 e1 Sig e2
         C sp, sx;
         sp.x = sp.y = sx.x = sx.y = 0;
 #pragma unroll
-        for (int i = 0; i < 3; i++)
-#pragma unroll
-            for (int j = 0; j < 3; j++) {
-                const T ep = (e1[i] * e1[j] - e2[i] * e2[j]) * is2;
-                const T ex = (e1[i] * e2[j] + e2[i] * e1[j]) * is2;
-                sp.x += ep * Sm[i][j].x;
-                sp.y += ep * Sm[i][j].y;
-                sx.x += ex * Sm[i][j].x;
-                sx.y += ex * Sm[i][j].y;
-            }
+        for (int i = 0; i < 3; i++) {
+            C a, b;   // (Sig e1)_i, (Sig e2)_i
+            a.x = Sm[i][0].x * e1[0] + Sm[i][1].x * e1[1] + Sm[i][2].x * e1[2];
+            a.y = Sm[i][0].y * e1[0] + Sm[i][1].y * e1[1] + Sm[i][2].y * e1[2];
+            b.x = Sm[i][0].x * e2[0] + Sm[i][1].x * e2[1] + Sm[i][2].x * e2[2];
+            b.y = Sm[i][0].y * e2[0] + Sm[i][1].y * e2[1] + Sm[i][2].y * e2[2];
+            sp.x += e1[i] * a.x - e2[i] * b.x;
+            sp.y += e1[i] * a.y - e2[i] * b.y;
+            sx.x += e1[i] * b.x;
+            sx.y += e1[i] * b.y;
+        }
+        const T is2 = T(0.70710678118654752440084436210484903928), s2 = T(1.41421356237309504880168872420969807857);
+        sp.x *= is2;
+        sp.y *= is2;
+        sx.x *= s2;
+        sx.y *= s2;
         // implicit midpoint: (I - dt/2 A) y' = (I + dt/2 A) y + dt (0, s), A = [[0,1],[-k2,-2Hc]]
         const T dt = p.dtau, hc = p.hc_half;
         const T m12 = -T(0.5) * dt, m21 = T(0.5) * dt * k2, m22 = T(1) + dt * hc;
@@ -183,16 +207,7 @@ __global__ void __launch_bounds__(256) k_solve(SolveParams<T> p)
     }
     // scalar slip chi (written over Sxx)
     {
-        C kks;
-        kks.x = kks.y = 0;
-#pragma unroll
-        for (int i = 0; i < 3; i++)
-#pragma unroll
-            for (int j = 0; j < 3; j++) {
-                kks.x += kt[i] * kt[j] * Sm[i][j].x;
-                kks.y += kt[i] * kt[j] * Sm[i][j].y;
-            }
-        const T f = -T(0.75) / (k2 * k2) * p.inv_n3;
+        const T f = -T(0.75) * ik2 * ik2 * p.inv_n3;
         C chi;
         chi.x = f * kks.x;
         chi.y = f * kks.y;
@@ -201,21 +216,11 @@ __global__ void __launch_bounds__(256) k_solve(SolveParams<T> p)
     // frame dragging B (written over F)
     if (p.b_space && !p.b_seed) {
         C *BS = reinterpret_cast<C *>(p.bstate);
-        C v[3];
-#pragma unroll
-        for (int l = 0; l < 3; l++) {
-            v[l].x = kt[0] * Sm[0][l].x + kt[1] * Sm[1][l].x + kt[2] * Sm[2][l].x;
-            v[l].y = kt[0] * Sm[0][l].y + kt[1] * Sm[1][l].y + kt[2] * Sm[2][l].y;
-        }
-        C kv;
-        kv.x = kt[0] * v[0].x + kt[1] * v[1].x + kt[2] * v[2].x;
-        kv.y = kt[0] * v[0].y + kt[1] * v[1].y + kt[2] * v[2].y;
-        const T ik2 = T(1) / k2;
         const T w = p.dtau_prev * ik2;
 #pragma unroll
         for (int j = 0; j < 3; j++) {
             // dtau W_j = dtau (-i) (v_j - kt_j kv / kt^2) / kt^2
-            const T px = v[j].x - kt[j] * kv.x * ik2, py = v[j].y - kt[j] * kv.y * ik2;
+            const T px = v[j].x - kt[j] * kks.x * ik2, py = v[j].y - kt[j] * kks.y * ik2;
             C b = inF[j];
             b.x = p.b_decay * b.x + w * py;
             b.y = p.b_decay * b.y - w * px;
@@ -229,13 +234,14 @@ __global__ void __launch_bounds__(256) k_solve(SolveParams<T> p)
         C kF;
         kF.x = kt[0] * F[0].x + kt[1] * F[1].x + kt[2] * F[2].x;
         kF.y = kt[0] * F[0].y + kt[1] * F[1].y + kt[2] * F[2].y;
-        const T ik2 = T(1) / k2;
         const T f = T(4) * ik2;
+        kF.x *= ik2;
+        kF.y *= ik2;
 #pragma unroll
         for (int i = 0; i < 3; i++) {
             C b;
-            b.x = f * (F[i].x - kt[i] * kF.x * ik2);
-            b.y = f * (F[i].y - kt[i] * kF.y * ik2);
+            b.x = f * (F[i].x - kt[i] * kF.x);
+            b.y = f * (F[i].y - kt[i] * kF.y);
             if (p.b_space) reinterpret_cast<C *>(p.bstate)[i * nh + e] = b;  // seeds the integration
             b.x *= p.inv_n3;
             b.y *= p.inv_n3;
