@@ -233,7 +233,7 @@ namespace {
 template <class T> pm_status do_update(Ctx &c)
 {
     StepScalars s = scalars(c, c.step, false);
-    launch_corr_kick<T>(c, s);
+    if (!s.newtonian) launch_corr_kick<T>(c, s);   // the Newtonian kick takes the correction along
     CKL("corr_kick");
     launch_kick_drift<T>(c, s);
     CKL("kick_drift");

@@ -156,7 +156,8 @@ struct Ctx {
 enum { EV_START = 0, EV_PROJECT = 1, EV_FWD_X = 2, EV_FWD_Y = 3, EV_FWD_Z = 4, EV_SOLVE = 5,
        EV_INV_Z = 6, EV_INV_Y = 7, EV_INV_X = 8, EV_KICK = 9, EV_SCAN = 10, EV_END = 11 };
 
-// FP32 to FP64 on the integer pipes (the conversion instruction runs on the FP64 pipe); the common range inline
+// FP32 to FP64 and back on the integer pipes (the conversion instructions run on the FP64 pipe), rounded to nearest
+// even; the common range inline
 static __device__ __noinline__ double f32_to_f64_any(float f) { return (double)f; }
 static __device__ __forceinline__ double f32_to_f64(float f)
 {
@@ -164,6 +165,15 @@ static __device__ __forceinline__ double f32_to_f64(float f)
     if (e - 1u < 254u)   // normal
         return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
     return (b << 1) == 0 ? __hiloint2double((int)b, 0) : f32_to_f64_any(f);
+}
+static __device__ __noinline__ float f64_to_f32_any(double d) { return (float)d; }
+static __device__ __forceinline__ float f64_to_f32(double d)
+{
+    const uint64_t b = (uint64_t)__double_as_longlong(d), m = b & 0x7fffffffffffffffull;
+    const uint32_t sign = (uint32_t)(b >> 32) & 0x80000000u, e = (uint32_t)(m >> 52);
+    if (e - 897u < 253u)   // a normal float, also after rounding
+        return __uint_as_float(sign | ((uint32_t)((m + 0x0fffffffull + ((m >> 29) & 1)) >> 29) - (896u << 23)));
+    return e == 0 ? __uint_as_float(sign) : f64_to_f32_any(d);
 }
 static __device__ __forceinline__ double widen(float f) { return f32_to_f64(f); }
 static __device__ __forceinline__ double widen(double f) { return f; }

@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(TC_THREADS)
 // offsets take 4 steps instead of 27 (slots of offsets 27..31 carry zero weights).  A fragments
 // are built from 4-byte (2-channel) shared-memory loads, B fragments once per thread from the
 // weights in global memory.  y = relu(conv(x, w) + b), BF16 [cell][16].
-__global__ void __launch_bounds__(CONV_THREADS, 3)
+__global__ void __launch_bounds__(CONV_THREADS, 4)
     k_conv_in2(const uint4 *__restrict__ x, const __nv_bfloat16 *__restrict__ w, const float *__restrict__ bias,
                __nv_bfloat16 *y, int n)
 {
@@ -755,7 +755,7 @@ __global__ void k_features(const T *R, const T *phi, double s0, double s1, __nv_
     const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= ncell) return;
     __nv_bfloat162 v[8];
-    v[0] = __floats2bfloat162_rn((float)((double)R[c] * s0), (float)((double)phi[c] * s1));
+    v[0] = __floats2bfloat162_rn(f64_to_f32(widen(R[c]) * s0), f64_to_f32(widen(phi[c]) * s1));
 #pragma unroll
     for (int k = 1; k < 8; k++) v[k] = __floats2bfloat162_rn(0.f, 0.f);
     uint4 *dst = reinterpret_cast<uint4 *>(x + 16 * c);
