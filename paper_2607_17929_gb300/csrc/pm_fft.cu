@@ -43,7 +43,13 @@ template <class T, int N, bool ZP = false, int V = 0> struct Lines {
     static constexpr int col0 = tuned ? sh.l : (sizeof(T) == 4 ? 8 : 4);
     static constexpr int col1 = col0 * TLC < 128 ? 128 / TLC : col0;
     static constexpr int col = col1 * TLC > 1024 ? 1024 / TLC : col1;
-    static constexpr int row = TL >= 256 ? 1 : 256 / TL;               // row pairs per block, x passes
+    // Row pairs per block of the x passes: 256 threads, 128 for sizes with a factor of three.  Those hold
+    // 24 points a thread, few warps fit an SM, and every exchange stops the whole block: smaller blocks
+    // leave others to run meanwhile (r2c / c2r, us, FP32 192^3: 354 / 206 with 256 threads, 316 / 185
+    // with 128; 288^3: 1277 / 758, 1196 / 721; 72^3: 32 / 38, 29 / 28; FP64 192^3: 3875 / 2112, 3631 /
+    // 1927; 64 threads gain no more).  With 8 points a thread it makes no difference (256^3: 458 / 279, 461 / 274).
+    static constexpr int row_threads = N % 3 == 0 && TL <= 128 ? 128 : 256;
+    static constexpr int row = TL >= 256 ? 1 : row_threads / TL;
     // resident blocks per SM the register allocation must allow
     static constexpr int tpsm = tuned ? sh.tpsm : (fftc::Geo<N>::P == 8 ? (sizeof(T) == 4 ? 1536 : 1024) : 0);
     static constexpr int col_min_blocks = tpsm / (TLC * col) > 0 ? tpsm / (TLC * col) : 1;
