@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(MTHREADS, 4) k_mass(const __grid_constant__ De
 // by two vertex lanes, and a vertex costs 36 products per particle of two cells.  Against 8^3 vertex tiles that
 // stage the charges of 9^3 cells and let each vertex gather from 8 cells (a record read 8 times, potentials, ranges
 // and a scan set up per tile), at 512^3 mixed 6.9 -> 4.0 ms early (sums of one plane in registers, 40 of them, so
-// 20 warps an SM), at 256^3 FP64 15.3 -> 8.8, late (192^3, z = 1, cells of up to 55 particles) 0.59 -> 0.56.  A cell per lane with its 8 corners in registers was faster early (3.4 ms) but ran as
+// 20 warps an SM), at 256^3 FP64 15.3 -> 8.0, late (192^3, z = 1, cells of up to 55 particles) 0.59 -> 0.56.  A cell per lane with its 8 corners in registers was faster early (3.4 ms) but ran as
 // long as its row's fullest cell (late 0.78 ms).
 // ---------------------------------------------------------------------------
 constexpr int DROWS = 10;                 // rows of cells of a tile along y, one warp each
@@ -368,7 +368,13 @@ __device__ __forceinline__ void charges(const DepParams<T> &p, const PartFU<T> &
     const T iE = rsqrt_t(e2);
     // E = a + u^2 / (E + a): the approximate E enters only the small term, so E keeps the
     // accuracy of a (the T^00 charge cancels against the background in R)
-    const T dE = div_t(u2, e2 * iE + p.a);
+    T dE;
+    if constexpr (sizeof(T) == 4) {
+        dE = div_t(u2, e2 * iE + p.a);
+    } else {   // a Newton step for dE (dE + 2 a) = u^2 from E - a: as accurate as the quotient, and fewer operations
+        const T E0 = e2 * iE, d0 = E0 - p.a;
+        dE = d0 - T(0.5) * (iE * (d0 * (E0 + p.a) - u2));
+    }
     const T E = p.a + dE;
     const T v2 = u2 * iE * iE;
     const T m = p.mass;
@@ -443,28 +449,29 @@ __device__ __forceinline__ void dep_epilogue(const DepParams<T> &p, const T *dn,
         k0.add(-nl * (T)p.inv_g);   // the k = 0 mode carries the mean of -Nl
     }
     reinterpret_cast<T *>(p.out.p[0])[g] = p.G * dS - p.c1 * ph - p.c2 * ch - nl;
-    // with dp = 2 dx d phi, dc = 2 dx d chi and e = 2 dp - dc (of phi + psi = 2 phi - chi):
-    //   2 TF[2 d_i phi d_j phi - d_i(phi + psi) d_j(phi + psi)] = N^2/2 TF[2 dp_i dp_j - e_i e_j]
-    T dp[3], dc[3], e[3];
+    // with dc = 2 dx d chi and b = 2 dx d psi (psi = phi - chi):
+    //   2 TF[2 d_i phi d_j phi - d_i(phi + psi) d_j(phi + psi)] = N^2/2 TF[dc_i dc_j - 2 b_i b_j]
+    T dc[3], b[3], hc[3], hb[3];
 #pragma unroll
     for (int d = 0; d < 3; d++) {
-        dp[d] = pu[d] - pd[d];
         dc[d] = cu[d] - cd[d];
-        e[d] = T(2) * dp[d] - dc[d];
+        b[d] = (pu[d] - pd[d]) - dc[d];
+        hc[d] = T(0.5) * p.n2 * dc[d];
+        hb[d] = p.n2 * b[d];
     }
     if (p.write_f) {
         const T f = (ph - phi2) * p.inv_dt2 * p.halfN;   // phi' / (2 dx)
 #pragma unroll
-        for (int d = 0; d < 3; d++) reinterpret_cast<T *>(p.out.p[1 + d])[g] = p.G * s[d] - f * (dp[d] - dc[d]);
+        for (int d = 0; d < 3; d++) reinterpret_cast<T *>(p.out.p[1 + d])[g] = p.G * s[d] - f * b[d];
     }
-    const T G4 = T(4) * p.G, h = T(0.5) * p.n2;
-    auto quad = [&](int i, int j) { return T(2) * dp[i] * dp[j] - e[i] * e[j]; };
+    const T G4 = T(4) * p.G;
+    auto quad = [&](int i, int j) { return hc[i] * dc[j] - hb[i] * b[j]; };
     const T qxx = quad(0, 0), qyy = quad(1, 1), tr3 = (qxx + qyy + quad(2, 2)) * T(1.0 / 3.0);
-    reinterpret_cast<T *>(p.out.p[4])[g] = G4 * s[3] - h * (qxx - tr3);
-    reinterpret_cast<T *>(p.out.p[5])[g] = G4 * s[4] - h * quad(0, 1);
-    reinterpret_cast<T *>(p.out.p[6])[g] = G4 * s[5] - h * quad(0, 2);
-    reinterpret_cast<T *>(p.out.p[7])[g] = G4 * s[6] - h * (qyy - tr3);
-    reinterpret_cast<T *>(p.out.p[8])[g] = G4 * s[7] - h * quad(1, 2);
+    reinterpret_cast<T *>(p.out.p[4])[g] = G4 * s[3] - (qxx - tr3);
+    reinterpret_cast<T *>(p.out.p[5])[g] = hb[0] * b[1] + (G4 * s[4] - hc[0] * dc[1]);
+    reinterpret_cast<T *>(p.out.p[6])[g] = hb[0] * b[2] + (G4 * s[5] - hc[0] * dc[2]);
+    reinterpret_cast<T *>(p.out.p[7])[g] = G4 * s[6] - (qyy - tr3);
+    reinterpret_cast<T *>(p.out.p[8])[g] = hb[1] * b[2] + (G4 * s[7] - hc[1] * dc[2]);
 }
 
 // A vertex lane's sums in one plane: of its own row of vertices and of the one at y + 1.
@@ -797,6 +804,7 @@ template <class T> struct KdParams {
     int N;
     int nrow, ntx, tz;   // cells of a tile along x, tiles along x, cells along z
     T a, a2, a_half2, inv_a_half, dt_kick, dt_drift_N, halfN;
+    T kick_N;            // dt_kick N/2
     const float *corr;   // force correction [cell][8] (CORR)
     T corr_scale;
 };
@@ -808,7 +816,7 @@ template <class T> struct KdParams {
 // What bounds it: the shared-memory pipe (a particle reads 32 vertices of 20 bytes, 5 of its 8 wavefronts) and, in
 // FP64, the FP64 pipe.  Against 8^3 tiles of 11^3 vertices, one search and three integer divisions per particle, and
 // the gradients of five fields kept in 20 registers (512^3 mixed 5.15 ms, 256^3 FP64 14.0, 288^3 Newtonian 0.52):
-// 3.6 ms, 11.1, 0.29.  Rows that hold more than 32 particles make their CTA's other warps wait (192^3 at z = 1:
+// 3.5 ms, 8.8, 0.29.  Rows that hold more than 32 particles make their CTA's other warps wait (192^3 at z = 1:
 // 0.33 -> 0.33).  Two planes between barriers, records staged in shared memory instead of registers, four CTAs of 64
 // registers an SM, two of 128: 0.58, 0.48, 0.61, 0.52 ms against 0.46 at 256^3 (the first two take L1 from the loads).
 constexpr int KROWS = 8, KD_THREADS = 32 * KROWS;
@@ -856,7 +864,9 @@ __device__ __forceinline__ void gather_phi(const T *const (&pl)[4], const T *Wx,
 //   s = (E + u^2/E) phi - E chi + u_j B_j      (coefficients c[5] of phi, chi, B of this particle),
 // so each of the 32 stencil vertices is first reduced to s (5 products) and only s is differenced and
 // interpolated, axis by axis (68 operations instead of the 280 of five fields' three gradients, and 3 sums
-// instead of 15).  g: 2 dx grad s; val: phi, chi, B at the particle.
+// instead of 15).  FP64 takes s/E in 4 operations a vertex, the small terms first, and multiplies the gradient by E:
+// 256^3 11.1 -> 8.8 ms, with carry_cells().  FP32 does not miss the operation and was slower with each order of the
+// four (0.46 -> 0.48 to 0.53 ms at 256^3).  g: 2 dx grad s (s/E); val: phi, chi, B at the particle.
 template <class T>
 __device__ __forceinline__ void gather_s(const Vtx4<T> *const (&sv)[4], const T *const (&sb)[4], const T (&c)[5], T fx, T fy,
                                          T fz, T (&g)[3], T (&val)[5])
@@ -873,7 +883,8 @@ __device__ __forceinline__ void gather_s(const Vtx4<T> *const (&sv)[4], const T 
             val[3] += w * a.by;
             val[4] += w * b;
         }
-        return c[0] * a.phi + c[1] * a.chi + (c[2] * a.bx + c[3] * a.by + c[4] * b);
+        if constexpr (sizeof(T) == 8) return c[0] * a.phi + (c[4] * b + (c[3] * a.by + (c[2] * a.bx - a.chi)));
+        else return c[0] * a.phi + c[1] * a.chi + (c[2] * a.bx + c[3] * a.by + c[4] * b);
     };
     auto line = [&](int kz, int v) {   // interpolated along x between kx = 1 and 2 (v: the vertex at kx = 1)
         const T s1 = at(kz, v, T(0), false), s2 = at(kz, v + 1, T(0), false);
@@ -938,6 +949,21 @@ __device__ __forceinline__ void add_correction(const KdParams<T> &p, int x, int 
 #pragma unroll
     for (int k = 0; k < 3; k++) u[k] += p.dt_kick * f * cv[k];
 }
+
+// An offset v that left its cell in FP64: f = v - floor(v) (0 and the next cell where that rounds to 1), carry the
+// cells crossed.  3 FP64 additions instead of floor, two comparisons and two conversions, all of which take the FP64
+// pipe: v + 1.5 2^52, rounded down, holds floor(v) in its low word.  False (f and carry of no use) at N cells or more.
+__device__ __forceinline__ bool carry_cells(double v, int N, double &f, int &carry)
+{
+    const double M = 6755399441055744.0;   // 1.5 2^52
+    const double r = __dadd_rd(v, M), g = v - (r - M);
+    const int lo = __double2loint(r), hi = __double2hiint(g) & 0x7fffffff;   // no -0
+    const bool one = hi >= 0x3ff00000;
+    f = __hiloint2double(one ? 0 : hi, one ? 0 : __double2loint(g));
+    carry = lo + one;
+    return __double2hiint(r) == 0x43380000 + (lo >> 31) && lo < N && lo > -N;
+}
+__device__ __forceinline__ bool carry_cells(float, int, float &, int &) { return false; }
 
 // CORR: with the force correction of a Newtonian context
 template <class T, bool NEWT, bool CORR = false>
@@ -1055,38 +1081,51 @@ __device__ __forceinline__ void kick_tile(const KdParams<T> &p, const int b)
                 const T u2 = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
                 const T e2 = p.a2 + u2;
                 const T iE = rsqrt_t(e2);
-                const T E = e2 * iE;
-                const T c[5] = {E + u2 * iE, -E, u[0], u[1], u[2]};
+                const T E = e2 * iE, by = sizeof(T) == 8 ? iE : T(1);
+                const T c[5] = {sizeof(T) == 8 ? T(1) + u2 * (iE * iE) : E + u2 * iE, -E, u[0] * by, u[1] * by, u[2] * by};
                 const Vtx4<T> *const pv[4] = {sv + slot[0], sv + slot[1], sv + slot[2], sv + slot[3]};
                 T val[5] = {0, 0, 0, 0, 0}, g[3];
                 gather_s(pv, pb, c, fx, fy, fz, g, val);
-                const T dtk = p.dt_kick * p.halfN;
+                const T dtk = sizeof(T) == 8 ? p.kick_N * E : p.kick_N;
 #pragma unroll
                 for (int d = 0; d < 3; d++) u[d] -= dtk * g[d];
                 const T v2 = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
                 const T iEd = rsqrt_t(p.a_half2 + v2);
-                const T fac = (T(1) + T(3) * val[0] - val[1] - val[0] * v2 * iEd * iEd) * iEd;
+                // (1 + (3 - v^2/E^2) phi - chi) / E, v^2 = E^2 - a^2
+                const T fac = ((T(1) - val[1]) + val[0] * (T(2) + p.a_half2 * (iEd * iEd))) * iEd;
 #pragma unroll
                 for (int d = 0; d < 3; d++) dx[d] = p.dt_drift_N * (u[d] * fac + val[2 + d]);
             }
             const T fo[3] = {fx, fy, fz};
             const int io[3] = {x0 + cx, y0 + w, z};
             int inew[3];
+            bool near = sizeof(T) == 8;
+            if constexpr (sizeof(T) == 8) {
 #pragma unroll
-            for (int d = 0; d < 3; d++) {
-                T f = fo[d] + dx[d];
-                T fl = floor(f);
-                f -= fl;
-                // a finite move is far below N cells; anything else (NaN, Inf) keeps the cell
-                int carry = (fabs(fl) < (T)N) ? (int)fl : 0;
-                if (f >= T(1)) {
-                    f = T(0);
-                    carry += 1;
+                for (int d = 0; d < 3; d++) {
+                    int carry;
+                    near &= carry_cells(fo[d] + dx[d], N, P.f[d], carry);
+                    inew[d] = wrapi(io[d] + carry, N);   // |carry| <= N
                 }
-                inew[d] = wrapi(io[d] + carry, N);   // |carry| <= N
-                P.f[d] = f;
-                P.u[d] = u[d];
             }
+            if (!near) {
+#pragma unroll
+                for (int d = 0; d < 3; d++) {
+                    T f = fo[d] + dx[d];
+                    T fl = floor(f);
+                    f -= fl;
+                    // a finite move is far below N cells; anything else (NaN, Inf) keeps the cell
+                    int carry = (fabs(fl) < (T)N) ? (int)fl : 0;
+                    if (f >= T(1)) {
+                        f = T(0);
+                        carry += 1;
+                    }
+                    inew[d] = wrapi(io[d] + carry, N);   // |carry| <= N
+                    P.f[d] = f;
+                }
+            }
+#pragma unroll
+            for (int d = 0; d < 3; d++) P.u[d] = u[d];
             P.cell = (inew[2] * N + inew[1]) * N + inew[0];
             p.part[i] = P;
             atomicAdd(&p.count[P.cell], 1);
@@ -1731,6 +1770,7 @@ template <class T> KdParams<T> kd_params(const Ctx &c, const StepScalars &s)
     p.dt_kick = (T)s.dtau_kick;
     p.dt_drift_N = (T)(s.dtau * c.N);
     p.halfN = (T)(0.5 * c.N);
+    p.kick_N = p.dt_kick * p.halfN;
     return p;
 }
 
