@@ -756,8 +756,8 @@ __global__ void __launch_bounds__(DEP_THREADS, dep_ctas<T, FULL>()) k_project(co
 }
 
 // The CIC density contrast of the P(k) diagnostic in FP32 contexts: the columns above with the weights and the sums
-// in two words.  In place of FP64 weights and atomics on the FP64 pipe: 256^3 0.98 (with clearing and the final
-// pass) -> 0.26 ms; FP64 contexts take k_project with unit mass, 1.0 -> 0.5.
+// in two words.  In place of FP64 weights and atomics on the FP64 pipe: 256^3 at z = 3 0.98 (with clearing and the
+// final pass) -> 0.55 ms.  FP64 contexts take k_project with unit mass.
 __global__ void __launch_bounds__(DEP_THREADS, 2) k_contrast(const __grid_constant__ DepParams<float> p)
 {
     deposit_tile<float, false, true>(p, blockIdx.x);
@@ -1151,7 +1151,7 @@ __global__ void __launch_bounds__(KD_THREADS, kd_ctas<T, NEWT>()) k_kick_drift(c
 }
 
 // The Newtonian kick with a force correction: one pass over the particles instead of k_corr_kick's before it
-// (256^3 mixed, both kicks: 0.50 -> 0.40 ms).
+// (256^3 mixed, both kicks: 0.50 -> 0.42 ms).
 template <class T>
 __global__ void __launch_bounds__(KD_THREADS, sizeof(T) == 4 ? 3 : 2) k_kick_corrected(const __grid_constant__ KdParams<T> p)
 {

@@ -37,7 +37,8 @@ template <class T> struct SolveParams {
     T b_decay, dtau_prev;
 };
 
-// FP64 takes the fewest operations (its pipe bounds the FP64 solve: 256^3 4.5 -> 3.2 ms); FP32, bound by memory, the
+// FP64 takes the fewest operations (its pipe bounds the FP64 solve: 256^3, bootstrap and one step, 4.7 -> 3.8 ms, with
+// the cheaper polarisations below); FP32, bound by memory, the
 // IEEE square root and quotients.
 __device__ __forceinline__ double inv_sqrt(double x) { return rsqrt(x); }
 __device__ __forceinline__ float inv_sqrt(float x) { return 1.f / sqrtf(x); }
