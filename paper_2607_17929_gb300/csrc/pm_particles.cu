@@ -15,6 +15,7 @@
 #include <type_traits>
 
 #include "pm_internal.cuh"
+#include "pm_rows.cuh"
 
 namespace pm {
 
@@ -587,7 +588,7 @@ template <class T, bool FULL, bool DEN> struct DepCol {
         B.zero();
         V *rv = reinterpret_cast<V *>(rec);            // [part][32]: weights dx = 0, dx = 1, T00 and the other charges
         const int base = wrapi(z, p.N) * (p.N * p.N) + row - 1;
-        for (int c0 = 0; c0 < r.total; c0 += 32) {
+        for_groups(r.total, [&](int c0) {
             const int i = c0 + lane;
             PartFU<T> P{};
             int cx = 0;                                // the cell's lower corner in the row's staged potentials
@@ -652,7 +653,7 @@ template <class T, bool FULL, bool DEN> struct DepCol {
             gather(max(r.prev - c0, 0), min(r.end - c0, 32), r.mid - c0);
             if (p.cyclic) gather(max(r.wrap - c0, 0), min(r.total - c0, 32), 32);   // lane 0: the row's last cell
             __syncwarp();
-        }
+        });
         T *xo = xch + (PAR * DROWS + w) * (32 * W) + lane;
         if (iz >= 0) {   // the sums for the row at y + 1
             xo[0] = A.t00[1].hi();
@@ -1017,7 +1018,7 @@ __device__ __forceinline__ void kick_tile(const KdParams<T> &p, const int b)
     // a row's first 32 records, ahead of their plane
     V nxt[PQ];
     auto fetch = [&](int s, int e) {
-        if (s + lane < e) {
+        if (lane < e - s) {   // not s + lane < e: that sum can pass 2^31 - 1
 #pragma unroll
             for (int q = 0; q < PQ; q++) nxt[q] = reinterpret_cast<const V *>(p.part + s + lane)[q];
         }
@@ -1049,8 +1050,10 @@ __device__ __forceinline__ void kick_tile(const KdParams<T> &p, const int b)
         for (int q = 0; q < PQ; q++) rec[q] = nxt[q];
         fetch(s1, e1);
         const int base = z * (N * N) + row;
-        for (int i = s0 + lane; i < e0; i += 32) {
-            if (i >= s0 + 32) {
+        for_groups(e0 - s0, [&](int c0) {
+            if (c0 + lane >= e0 - s0) return;
+            const int i = s0 + c0 + lane;
+            if (c0 > 0) {
 #pragma unroll
                 for (int q = 0; q < PQ; q++) rec[q] = reinterpret_cast<const V *>(p.part + i)[q];
             }
@@ -1129,7 +1132,7 @@ __device__ __forceinline__ void kick_tile(const KdParams<T> &p, const int b)
             P.cell = (inew[2] * N + inew[1]) * N + inew[0];
             p.part[i] = P;
             atomicAdd(&p.count[P.cell], 1);
-        }
+        });
         // plane z + 3 into the slot of plane z - 2, last read before the barrier of the plane before
         if (iz + 1 < nz) keep(sc + 4 >= KRING ? sc + 4 - KRING : sc + 4);
         __syncthreads();
