@@ -163,17 +163,17 @@ __device__ __forceinline__ T hc_remainder(T ph, const T (&up)[3], const T (&dn)[
 // ---------------------------------------------------------------------------
 constexpr int MT = 8, MR = MT + 1, MCELLS = MR * MR * MR, MTHREADS = MT * MT * MT;
 constexpr int MOWN = 8;     // particles of two cells that their thread stages itself
-constexpr int MCAP = 960;   // particles staged at a time (a nearly uniform load of one per cell has 729)
 
-struct MassSmem {
+template <class I> struct MassSmem {
     float4 rec[MCAP];                         // f
-    int off[MCELLS + 1];                      // exclusive scan of the cells' counts
-    int warp[MTHREADS / 32];
+    I off[MCELLS + 1];                        // exclusive scan of the cells' counts
+    I warp[MTHREADS / 32];
 };
 
-__device__ __forceinline__ void mass_tile(const DepParams<float> &p, const int b)
+// I: type of the tile's offsets (mass_wide)
+template <class I> __device__ __forceinline__ void mass_tile(const DepParams<float> &p, const int b)
 {
-    __shared__ MassSmem sm;
+    __shared__ MassSmem<I> sm;
     const int N = p.N, nt = N / MT, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int x0 = (b % nt) * MT, y0 = ((b / nt) % nt) * MT, z0 = (b / (nt * nt)) * MT;
     // first particle and count of cells 2 tid and 2 tid + 1, then the exclusive scan of the counts
@@ -188,22 +188,22 @@ __device__ __forceinline__ void mass_tile(const DepParams<float> &p, const int b
             n[q] = __ldg(p.start + g + 1) - s[q];
         }
     }
-    int inc = n[0] + n[1];
+    I inc = (I)n[0] + n[1];
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, inc, o);
+        const I v = __shfl_up_sync(0xffffffffu, inc, o);
         if (lane >= o) inc += v;
     }
     if (lane == 31) sm.warp[wid] = inc;
     __syncthreads();
-    int before = 0, total = 0;
+    I before = 0, total = 0;
 #pragma unroll
     for (int w = 0; w < MTHREADS / 32; w++) {
-        const int v = sm.warp[w];
+        const I v = sm.warp[w];
         before += w < wid ? v : 0;
         total += v;
     }
-    const int e = before + inc - n[0] - n[1];
+    const I e = before + inc - n[0] - n[1];
     if (2 * tid <= MCELLS) sm.off[2 * tid] = e;
     if (2 * tid + 1 <= MCELLS) sm.off[2 * tid + 1] = e + n[0];
     __syncthreads();
@@ -211,8 +211,8 @@ __device__ __forceinline__ void mass_tile(const DepParams<float> &p, const int b
     const int ox = tid % MT, oy = (tid / MT) % MT, oz = tid / (MT * MT);
     Acc<float> acc;
     acc.zero();
-    for (int lo = 0; lo < total; lo += MCAP) {
-        const int hi = min(total, lo + MCAP);
+    for (I lo = 0; lo < total; lo += MCAP) {
+        const I hi = min(total, lo + MCAP);
         // each thread stages the particles of its two cells, MOWN at most; the warp
         // together stages what is left in crowded cells
         auto stage = [&](int first0, int n0, int first1, int k, int to) {
@@ -220,15 +220,20 @@ __device__ __forceinline__ void mass_tile(const DepParams<float> &p, const int b
             const float2 xy = __ldg(reinterpret_cast<const float2 *>(q + 2));
             sm.rec[to] = make_float4(xy.x, xy.y, __ldg(q + 4), 0.f);
         };
-        const int k0 = max(lo - e, 0), k1 = min(n[0] + n[1], hi - e), ko = min(k1, k0 + MOWN);
+        // its share k0 .. k1 - 1 of the pair's particles (at most n_part, so that an int holds k but not k + 32)
+        const I m = (I)n[0] + n[1];
+        const int k0 = (int)min(max(lo - e, I(0)), m), k1 = (int)max(min(m, hi - e), I(0));
+        const int ko = k0 + min(max(k1 - k0, 0), MOWN);
 #pragma unroll 1
-        for (int k = k0; k < ko; k++) stage(s[0], n[0], s[1], k, e + k - lo);
+        for (int k = k0; k < ko; k++) stage(s[0], n[0], s[1], k, (int)(e - lo) + k);
         for (unsigned left = __ballot_sync(0xffffffffu, ko < k1); left; left &= left - 1) {
             const int o = __ffs(left) - 1;
             const int f0 = __shfl_sync(0xffffffffu, s[0], o), m0 = __shfl_sync(0xffffffffu, n[0], o),
-                      f1 = __shfl_sync(0xffffffffu, s[1], o), to = __shfl_sync(0xffffffffu, e, o) - lo,
-                      end = __shfl_sync(0xffffffffu, k1, o);
-            for (int k = __shfl_sync(0xffffffffu, ko, o) + lane; k < end; k += 32) stage(f0, m0, f1, k, to + k);
+                      f1 = __shfl_sync(0xffffffffu, s[1], o), to = (int)(__shfl_sync(0xffffffffu, e, o) - lo),
+                      k = __shfl_sync(0xffffffffu, ko, o), end = __shfl_sync(0xffffffffu, k1, o);
+            for_groups(end - k, [&](int c) {
+                if (c + lane < end - k) stage(f0, m0, f1, k + c + lane, to + k + c + lane);
+            });
         }
         __syncthreads();
         // vertex o receives from cells o - d, d in {0,1}^3, weight (d ? f : 1 - f) per axis; the x-neighbours
@@ -238,10 +243,10 @@ __device__ __forceinline__ void mass_tile(const DepParams<float> &p, const int b
 #pragma unroll
             for (int dy = 0; dy < 2; dy++) {
                 const int ts = ox + MR * ((oy + 1 - dy) + MR * (oz + 1 - dz));   // cell with dx = 1
-                const int mid = sm.off[ts + 1];                                  // first particle with dx = 0
-                const int je = min(sm.off[ts + 2], hi);
-                for (int j = max(sm.off[ts], lo); j < je; j++) {
-                    const float4 f = sm.rec[j - lo];
+                const I mid = sm.off[ts + 1];                                  // first particle with dx = 0
+                const I je = min(sm.off[ts + 2], hi);
+                for (I j = max(sm.off[ts], lo); j < je; j++) {
+                    const float4 f = sm.rec[(int)(j - lo)];
                     const float wyz = (dy ? f.y : 1.f - f.y) * (dz ? f.z : 1.f - f.z);
                     const float w = (j < mid ? f.x : 1.f - f.x) * wyz;
                     acc.add(mulr(w, p.mass));
@@ -254,7 +259,10 @@ __device__ __forceinline__ void mass_tile(const DepParams<float> &p, const int b
     reinterpret_cast<float *>(p.out.p[0])[go] = p.G * ((acc.hi() - p.rb_hi) + (acc.lo() - p.rb_lo));
 }
 
-__global__ void __launch_bounds__(MTHREADS, 4) k_mass(const __grid_constant__ DepParams<float> p) { mass_tile(p, blockIdx.x); }
+template <class I> __global__ void __launch_bounds__(MTHREADS, 4) k_mass(const __grid_constant__ DepParams<float> p)
+{
+    mass_tile<I>(p, blockIdx.x);
+}
 
 // ---------------------------------------------------------------------------
 // Deposit.  A CTA owns the vertices [x0, x0 + nrow) x [y0, y0 + ncol) x [z0, z0 + tz) and visits the cells
@@ -782,11 +790,12 @@ __global__ void __launch_bounds__(DEP_THREADS, dep_ctas<T, FULL>()) k_project_ba
     deposit_tile<T, FULL>(q.box[i], (int)blockIdx.x - q.first[i]);
 }
 
+template <class I>
 __global__ void __launch_bounds__(MTHREADS, 4) k_mass_batch(const __grid_constant__ DepBatch<float> q)
 {
     int i = 0;
     while (i + 1 < q.nbox && (int)blockIdx.x >= q.first[i + 1]) i++;
-    mass_tile(q.box[i], (int)blockIdx.x - q.first[i]);
+    mass_tile<I>(q.box[i], (int)blockIdx.x - q.first[i]);
 }
 
 // ---------------------------------------------------------------------------
@@ -1717,7 +1726,7 @@ void launch_project(Ctx &c, const StepScalars &s)
         dep_attrs<T, false>();
         k_project<T, false><<<dep_ntiles(p), DEP_THREADS, dep_smem<T, false, false>(), c.stream>>>(p);
     } else if constexpr (sizeof(T) == 4) {
-        k_mass<<<dep_ntiles(p), MTHREADS, 0, c.stream>>>(p);
+        (mass_wide(c.N, c.np) ? k_mass<int64_t> : k_mass<int>)<<<dep_ntiles(p), MTHREADS, 0, c.stream>>>(p);
     }
     c.launches++;
 }
@@ -1741,7 +1750,9 @@ void launch_project_batch(Ctx *const *cs, const StepScalars *ss, int n, bool ful
             dep_attrs<T, true>();
             k_project_batch<T, true><<<q.first[nb], DEP_THREADS, dep_smem<T, true, false>(), st>>>(q);
         } else if constexpr (sizeof(T) == 4) {
-            k_mass_batch<<<q.first[nb], MTHREADS, 0, st>>>(q);
+            bool wide = false;
+            for (int i = 0; i < nb; i++) wide |= mass_wide(cs[b0 + i]->N, cs[b0 + i]->np);
+            (wide ? k_mass_batch<int64_t> : k_mass_batch<int>)<<<q.first[nb], MTHREADS, 0, st>>>(q);
         } else {
             dep_attrs<T, false>();
             k_project_batch<T, false><<<q.first[nb], DEP_THREADS, dep_smem<T, false, false>(), st>>>(q);

@@ -40,3 +40,23 @@ def test_groups_of_a_row(walk, n):
     groups = (n + 31) // 32
     assert walk(n) == f"{groups} {32 * (groups - 1)} 0"
     assert n == 0 or 32 * (groups - 1) + 31 < 2 ** 31
+
+
+def test_offsets_of_a_mass_tile_fit_their_type(tmp_path):
+    """Where the mass deposit counts a tile's particles in 32 bits, the count and the end of its last chunk fit."""
+    (tmp_path / "m.cpp").write_text("""
+#include <cstdio>
+#include <cstdlib>
+#include "pm_rows.cuh"
+int main(int, char **v) { printf("%d %d", (int)pm::mass_wide(atoi(v[1]), atoll(v[2])), pm::MCAP); }
+""")
+    exe = str(tmp_path / "m")
+    subprocess.check_call(["g++", "-std=c++20", "-I", os.path.join(ROOT, "paper_2607_17929_gb300", "csrc"),
+                           str(tmp_path / "m.cpp"), "-o", exe])
+    for n in (8, 16, 24, 128, 1024):
+        for np_ in (1, 512, 2 ** 27, 2 ** 28 - 200, 2 ** 28 - 1, 2 ** 28, 2 ** 31 - 2000, 2 ** 31 - 900, 2 ** 31 - 1):
+            wide, cap = map(int, subprocess.check_output([exe, str(n), str(np_)], text=True).split())
+            # cells x0 - 1 .. x0 + 7 along an axis: on 8 cells one of them is there twice
+            most = np_ * (8 if n == 8 else 1)
+            assert wide or most + cap < 2 ** 31, (n, np_)
+            assert not wide or most > 2 ** 31 - 2000, (n, np_)   # only where it is needed
