@@ -197,24 +197,23 @@ k_c2r_fast(const __grid_constant__ Ptrs in, const __grid_constant__ Ptrs out, co
 template <class T, int N> struct FastPasses {
     static void attrs()
     {
-        static std::atomic<uint64_t> done{0};
-        if (!first_on_device(done)) return;
-        auto set = [](auto k, size_t b) { cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b); };
-        set_col<0>();
-        if constexpr (Lines<T, N>::tuned) {
-            set_col<1>();
-            set_col<2>();
-        }
-        set(k_r2c_fast<T, N>, row_fast_smem<T, N>());
-        set(k_c2r_fast<T, N>, row_fast_smem<T, N>());
+        static DeviceOnce once;
+        once_on_device(once, [] {
+            set_col<0>();
+            if constexpr (Lines<T, N>::tuned) {
+                set_col<1>();
+                set_col<2>();
+            }
+            allow_smem(k_r2c_fast<T, N>, row_fast_smem<T, N>());
+            allow_smem(k_c2r_fast<T, N>, row_fast_smem<T, N>());
+        });
     }
     template <int V> static void set_col()
     {
-        auto set = [](auto k, size_t b) { cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b); };
-        set(k_col_fast<T, N, -1, false, V>, col_fast_smem<T, N, false, V>());
-        set(k_col_fast<T, N, 1, false, V>, col_fast_smem<T, N, false, V>());
-        set(k_col_fast<T, N, -1, true, V>, col_fast_smem<T, N, true, V>());
-        set(k_col_fast<T, N, 1, true, V>, col_fast_smem<T, N, true, V>());
+        allow_smem(k_col_fast<T, N, -1, false, V>, col_fast_smem<T, N, false, V>());
+        allow_smem(k_col_fast<T, N, 1, false, V>, col_fast_smem<T, N, false, V>());
+        allow_smem(k_col_fast<T, N, -1, true, V>, col_fast_smem<T, N, true, V>());
+        allow_smem(k_col_fast<T, N, 1, true, V>, col_fast_smem<T, N, true, V>());
     }
     template <bool ZP, int V>
     static void cols_t(Ctx &c, int nf, const Ptrs &p, int dir)

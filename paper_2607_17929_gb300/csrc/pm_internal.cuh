@@ -4,11 +4,11 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <atomic>
 #include <string>
 #include <vector>
 
 #include "../../include/pm.h"
+#include "pm_once.cuh"
 
 namespace pm {
 
@@ -178,14 +178,17 @@ static __device__ __forceinline__ float f64_to_f32(double d)
 static __device__ __forceinline__ double widen(float f) { return f32_to_f64(f); }
 static __device__ __forceinline__ double widen(double f) { return f; }
 
-// True the first time it is called with `mask` on the current device (for per-device one-time set-up
-// such as kernel attributes; a repeated set-up from a racing thread is harmless).
-inline bool first_on_device(std::atomic<uint64_t> &mask)
+// set-up of the current device, such as kernel attributes, unless it was done
+template <class F> void once_on_device(DeviceOnce &once, F &&set)
 {
-    int d = 0;
+    int d = -1;
     cudaGetDevice(&d);
-    const uint64_t bit = 1ull << (d & 63);
-    return (mask.fetch_or(bit) & bit) == 0;
+    once(d, set);
+}
+// raises kernel k's dynamic shared memory to `bytes`
+template <class K> void allow_smem(K k, size_t bytes)
+{
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 // ---------------------------------------------------------------------------

@@ -895,9 +895,8 @@ template <bool RELU, bool OUTF32, bool MASK = false>
 void launch_conv_tc(const uint4 *x, const uint4 *w, const float *b, void *y, int n, cudaStream_t st,
                     const uint4 *mact = nullptr, float *db = nullptr)
 {
-    static std::atomic<uint64_t> done{0};
-    if (first_on_device(done))
-        cudaFuncSetAttribute(k_conv_tc<RELU, OUTF32, MASK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
+    static DeviceOnce once;
+    once_on_device(once, [] { allow_smem(k_conv_tc<RELU, OUTF32, MASK>, TC_SMEM); });
     const int ntiles = (n / TCX) * (n / TCY) * (n / TCZ);
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
@@ -957,8 +956,8 @@ int dw_blocks(int n)
 
 void launch_conv_dw(const uint4 *x, const uint4 *g, float *dw, int n, cudaStream_t st)
 {
-    static std::atomic<uint64_t> done{0};
-    if (first_on_device(done)) cudaFuncSetAttribute(k_conv_dw, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DW_SMEM);
+    static DeviceOnce once;
+    once_on_device(once, [] { allow_smem(k_conv_dw, DW_SMEM); });
     k_conv_dw<<<dw_blocks(n), 32 * DW_WARPS, DW_SMEM, st>>>(x, g, dw, n);
 }
 

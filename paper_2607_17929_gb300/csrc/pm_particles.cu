@@ -1699,13 +1699,11 @@ template <class T> DepParams<T> dep_params(const Ctx &c, const StepScalars &s)
 
 template <class T, bool FULL> void dep_attrs()
 {
-    static std::atomic<uint64_t> attr{0};
-    if (first_on_device(attr)) {
-        cudaFuncSetAttribute(k_project<T, FULL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dep_smem<T, FULL, false>());
-        if constexpr (sizeof(T) == 8 || FULL)
-            cudaFuncSetAttribute(k_project_batch<T, FULL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)dep_smem<T, FULL, false>());
-    }
+    static DeviceOnce once;
+    once_on_device(once, [] {
+        allow_smem(k_project<T, FULL>, dep_smem<T, FULL, false>());
+        if constexpr (sizeof(T) == 8 || FULL) allow_smem(k_project_batch<T, FULL>, dep_smem<T, FULL, false>());
+    });
 }
 
 // the mixed Newtonian mode takes k_mass
@@ -1801,11 +1799,11 @@ template <class T> int kd_ntiles(const KdParams<T> &p) { return p.ntx * (p.N / K
 
 template <class T, bool NEWT> void kd_attrs()
 {
-    static std::atomic<uint64_t> attr{0};
-    if (first_on_device(attr)) {
-        cudaFuncSetAttribute(k_kick_drift<T, NEWT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kd_smem<T, NEWT>());
-        cudaFuncSetAttribute(k_kick_batch<T, NEWT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kd_smem<T, NEWT>());
-    }
+    static DeviceOnce once;
+    once_on_device(once, [] {
+        allow_smem(k_kick_drift<T, NEWT>, kd_smem<T, NEWT>());
+        allow_smem(k_kick_batch<T, NEWT>, kd_smem<T, NEWT>());
+    });
 }
 
 template <class T>
@@ -1813,9 +1811,8 @@ void launch_kick_drift(Ctx &c, const StepScalars &s)
 {
     KdParams<T> p = kd_params<T>(c, s);
     if (s.newtonian && c.corr) {
-        static std::atomic<uint64_t> attr{0};
-        if (first_on_device(attr))
-            cudaFuncSetAttribute(k_kick_corrected<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kd_smem<T, true>());
+        static DeviceOnce once;
+        once_on_device(once, [] { allow_smem(k_kick_corrected<T>, kd_smem<T, true>()); });
         p.corr = static_cast<const float *>(c.corr);
         p.corr_scale = (T)c.corr_scale;
         k_kick_corrected<T><<<kd_ntiles(p), KD_THREADS, kd_smem<T, true>(), c.stream>>>(p);
@@ -1988,9 +1985,9 @@ void launch_density(Ctx &c, void *real_out)
     p.magic = (T)std::ldexp(1.5, std::ilogb(std::max(1.0, mean)) + 1 - 13 + 23);
     const int nt = p.ntx * p.nty * ((p.N + p.tz - 1) / p.tz);
     if constexpr (sizeof(T) == 4) {
-        static std::atomic<uint64_t> attr{0};
-        constexpr int bytes = (int)dep_smem<float, false, true>();
-        if (first_on_device(attr)) cudaFuncSetAttribute(k_contrast, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        static DeviceOnce once;
+        constexpr size_t bytes = dep_smem<float, false, true>();
+        once_on_device(once, [] { allow_smem(k_contrast, bytes); });
         k_contrast<<<nt, DEP_THREADS, bytes, c.stream>>>(p);
     } else {
         dep_attrs<T, false>();
