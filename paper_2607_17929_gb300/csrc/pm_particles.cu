@@ -22,16 +22,19 @@ namespace pm {
 namespace {
 
 
-// Per-cell accumulator of the T^00 charge, whose cell sums cancel against the
-// uniform background in R.  FP64: plain double.  Mixed: float-float with
-// Knuth's TwoSum, so a cell sum keeps about 48 significant bits.  The other
+// Accumulator of the T^00 charge, whose sums cancel against the uniform
+// background in R.  FP64: plain double.  Mixed: float-float with Knuth's
+// TwoSum, which loses nothing of a term whatever its size and the sum's, and
+// the roundings of the high word summed up in the low one: about 48
+// significant bits, and as many less as that word's own roundings come to
+// (n terms: at most 2^-24 of their share, n 2^-24 of the sum).  The other
 // components have no such cancellation and are summed in the field type.
 template <class T> struct Acc;
 template <> struct Acc<double> {
     double s;
     __device__ __forceinline__ void zero() { s = 0.0; }
     __device__ __forceinline__ void add(double x) { s += x; }
-    __device__ __forceinline__ void add_product(double a, double b, double) { s = fma(a, b, s); }
+    __device__ __forceinline__ void add_product(double a, double b) { s = fma(a, b, s); }
     __device__ __forceinline__ double hi() const { return s; }
     __device__ __forceinline__ double lo() const { return 0.0; }
 };
@@ -46,22 +49,11 @@ template <> struct Acc<float> {
         s = t;
         c = __fadd_rn(c, e);
     }
-    // += a b.  The magic number M = 1.5 2^23 U rounds the product to a multiple of U, which sums up exactly in s
-    // below 2^24 U; the exact rest (at most U / 2) goes to c.  Five operations after the product instead of the
-    // seven of add().
-    __device__ __forceinline__ void add_product(float a, float b, float M)
+    __device__ __forceinline__ void add_product(float a, float b) { add(__fmul_rn(a, b)); }
+    __device__ __forceinline__ void add_two(float x, float lo)
     {
-        const float x = __fmul_rn(a, b);
-        const float h = __fsub_rn(__fadd_rn(x, M), M);
-        s = __fadd_rn(s, h);
-        c = __fadd_rn(c, __fsub_rn(x, h));
-    }
-    // += x + lo
-    __device__ __forceinline__ void add_split(float x, float lo, float M)
-    {
-        const float h = __fsub_rn(__fadd_rn(x, M), M);
-        s = __fadd_rn(s, h);
-        c = __fadd_rn(c, __fadd_rn(__fsub_rn(x, h), lo));
+        add(x);
+        c = __fadd_rn(c, lo);
     }
     __device__ __forceinline__ float hi() const { return s; }
     __device__ __forceinline__ float lo() const { return c; }
@@ -95,7 +87,6 @@ template <class T> struct DepParams {
     int cyclic;      // one tile along x: the cell x0 - 1 is the row's last
     int newtonian;
     T a, a2, mass;
-    T magic;         // of Acc<float>::add_product: U = 2^-13 of a power of two above a particle's charge and the mean load
     T G;             // 4piG a^-2 N^3 (Newtonian: 4piG a^-1 N^3)
     T rb_hi, rb_lo;  // expected per-vertex charge sum of a uniform load, float-float split
     T c1, c2;        // 3Hc/dtau_{n-1}, 3Hc^2
@@ -634,17 +625,17 @@ template <class T, bool FULL, bool DEN> struct DepCol {
                     for (int k = 0; k < 4 / VT; k++) unpackv(v[32 * k], wn + VT * k);
                     if constexpr (DEN) {
                         unpackv(v[64], qn);
-                        A.t00[0].add_split(wn[0], qn[0], p.magic);
-                        A.t00[1].add_split(wn[1], qn[1], p.magic);
-                        B.t00[0].add_split(wn[2], qn[2], p.magic);
-                        B.t00[1].add_split(wn[3], qn[3], p.magic);
+                        A.t00[0].add_two(wn[0], qn[0]);
+                        A.t00[1].add_two(wn[1], qn[1]);
+                        B.t00[0].add_two(wn[2], qn[2]);
+                        B.t00[1].add_two(wn[3], qn[3]);
                         continue;
                     }
                     const T t = r0[n];
-                    A.t00[0].add_product(wn[0], t, p.magic);
-                    A.t00[1].add_product(wn[1], t, p.magic);
-                    B.t00[0].add_product(wn[2], t, p.magic);
-                    B.t00[1].add_product(wn[3], t, p.magic);
+                    A.t00[0].add_product(wn[0], t);
+                    A.t00[1].add_product(wn[1], t);
+                    B.t00[0].add_product(wn[2], t);
+                    B.t00[1].add_product(wn[3], t);
                     if constexpr (FULL) {
 #pragma unroll
                         for (int k = 0; k < 8 / VT; k++) unpackv(rv[32 * (8 / VT + k) + n], qn + VT * k);
@@ -679,14 +670,18 @@ template <class T, bool FULL, bool DEN> struct DepCol {
         rn = range(nb);
         if (out) {
             const T *xi = xo - 32 * W;
+            Acc<T> S = A.t00[0], S2;
+            S2.s = xi[0];
+            if constexpr (sizeof(T) == 4) S2.c = xi[32];
+            acc_merge(S, S2);
             // R: the uniform background a*Omega_m is removed before rounding
-            T dS = (A.t00[0].hi() + xi[0]) - p.rb_hi;
-            if constexpr (sizeof(T) == 4) dS += (A.t00[0].lo() + xi[32]) - p.rb_lo;
+            const T dS = (S.hi() - p.rb_hi) + (S.lo() - p.rb_lo);
             const int g = cells + lane;
             if constexpr (DEN) {
                 // the contrast N^3 / n_part (S - n_part / N^3) in two words
-                const float h = (A.t00[0].hi() + xi[0]) - p.rb_hi, l = (A.t00[0].lo() + xi[32]) - p.rb_lo;
-                const float sum = __fadd_rn(h, l), low = __fsub_rn(l, __fsub_rn(sum, h)), x = __fmul_rn(p.G, sum);
+                S.add(-p.rb_hi);
+                const float l = S.lo() - p.rb_lo;
+                const float sum = __fadd_rn(S.hi(), l), low = __fsub_rn(l, __fsub_rn(sum, S.hi())), x = __fmul_rn(p.G, sum);
                 reinterpret_cast<T *>(p.out.p[0])[g] = x + (__fmaf_rn(p.G, sum, -x) + (p.G * low + p.c1 * sum));
             } else if constexpr (!FULL) {
                 reinterpret_cast<T *>(p.out.p[0])[g] = p.G * dS;
@@ -1683,8 +1678,6 @@ template <class T> DepParams<T> dep_params(const Ctx &c, const StepScalars &s)
     }
     p.rb_hi = (T)rb;
     p.rb_lo = (T)(rb - (double)p.rb_hi);
-    const double top = std::max(s.newtonian ? s.mass : s.a * s.mass, rb);   // sums stay exact up to 2048 of it
-    p.magic = (T)std::ldexp(1.5, std::ilogb(top) + 1 - 13 + 23);
     p.c1 = (T)s.c_phi_dt;
     p.c2 = (T)s.c_phi_h2;
     p.inv_dt2 = (T)s.inv_dtau_prev2;
@@ -1982,7 +1975,6 @@ void launch_density(Ctx &c, void *real_out)
     p.c1 = (T)(q - (double)p.G);
     p.rb_hi = (T)mean;
     p.rb_lo = (T)(mean - (double)p.rb_hi);
-    p.magic = (T)std::ldexp(1.5, std::ilogb(std::max(1.0, mean)) + 1 - 13 + 23);
     const int nt = p.ntx * p.nty * ((p.N + p.tz - 1) / p.tz);
     if constexpr (sizeof(T) == 4) {
         static DeviceOnce once;
