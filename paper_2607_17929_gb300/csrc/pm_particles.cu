@@ -761,7 +761,7 @@ __global__ void __launch_bounds__(DEP_THREADS, dep_ctas<T, FULL>()) k_project(co
 
 // The CIC density contrast of the P(k) diagnostic in FP32 contexts: the columns above with the weights and the sums
 // in two words.  In place of FP64 weights and atomics on the FP64 pipe: 256^3 at z = 3 0.98 (with clearing and the
-// final pass) -> 0.55 ms.  FP64 contexts take k_project with unit mass.
+// final pass) -> 0.55 ms.  FP64 contexts take k_density_acc.
 __global__ void __launch_bounds__(DEP_THREADS, 2) k_contrast(const __grid_constant__ DepParams<float> p)
 {
     deposit_tile<float, false, true>(p, blockIdx.x);
@@ -1594,6 +1594,30 @@ __global__ void __launch_bounds__(256) k_store(const Particle<T> *byid, int64_t 
     }
 }
 
+// CIC density contrast N^3 / n_part sum w - 1 of FP64 contexts, a particle per thread.  Bound by the FP64 atomics, which
+// take about as long whatever the cells hold: 128^3 P(k) 0.38 ms at z = 50 and at z = 1, 0.49 with a tenth of the mass in
+// cells of 10^4.  The columns of the deposit, whose warps wait for their fullest cell on the FP64 pipe, took 0.42, 0.65
+// and 4.3.
+__global__ void k_density_acc(const Particle<double> *part, int64_t np, int N, double q, double *rho)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= np) return;
+    const Particle<double> P = part[i];
+    const int ix = P.cell % N, iy = (P.cell / N) % N, iz = P.cell / (N * N);
+#pragma unroll
+    for (int v = 0; v < 8; v++) {
+        const int dx = v & 1, dy = v >> 1 & 1, dz = v >> 2;
+        const double w = (dx ? P.f[0] : 1 - P.f[0]) * (dy ? P.f[1] : 1 - P.f[1]) * (dz ? P.f[2] : 1 - P.f[2]);
+        atomicAdd(&rho[((int64_t)wrapi(iz + dz, N) * N + wrapi(iy + dy, N)) * N + wrapi(ix + dx, N)], q * w);
+    }
+}
+
+__global__ void k_density_fin(double *rho, int64_t n)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) rho[i] -= 1.0;
+}
+
 template <class T> __global__ void k_to_f64(const T *s, double *d, int64_t n)
 {
     // four values a thread: with one, starting the blocks takes longer than the copy
@@ -1959,32 +1983,34 @@ void launch_store_packed(Ctx &c, pm_packed_particle *out, int64_t first, int64_t
 }
 
 // CIC mass density contrast delta = rho / omega_m - 1
-template <class T>
-void launch_density(Ctx &c, void *real_out)
+template <> void launch_density<double>(Ctx &c, void *real_out)
 {
-    DepParams<T> p{};
-    p.part = reinterpret_cast<const Particle<T> *>(c.part[c.cur]);
+    double *rho = static_cast<double *>(real_out);
+    cudaMemsetAsync(rho, 0, sizeof(double) * c.nc, c.stream);
+    k_density_acc<<<nblk(c.np, 256), 256, 0, c.stream>>>(reinterpret_cast<const Particle<double> *>(c.part[c.cur]), c.np, c.N,
+                                                         (double)c.nc / (double)c.np, rho);
+    k_density_fin<<<nblk(c.nc, 256), 256, 0, c.stream>>>(rho, c.nc);
+}
+
+template <> void launch_density<float>(Ctx &c, void *real_out)
+{
+    DepParams<float> p{};
+    p.part = reinterpret_cast<const Particle<float> *>(c.part[c.cur]);
     p.start = c.start;
     p.out.p[0] = real_out;
     p.N = c.N;
     p.newtonian = 1;
-    p.mass = T(1);
+    p.mass = 1.f;
     dep_tiles(p, false, c.dep_shape);
     const double mean = (double)c.np / (double)c.nc, q = (double)c.nc / (double)c.np;
-    p.G = (T)q;
-    p.c1 = (T)(q - (double)p.G);
-    p.rb_hi = (T)mean;
-    p.rb_lo = (T)(mean - (double)p.rb_hi);
-    const int nt = p.ntx * p.nty * ((p.N + p.tz - 1) / p.tz);
-    if constexpr (sizeof(T) == 4) {
-        static DeviceOnce once;
-        constexpr size_t bytes = dep_smem<float, false, true>();
-        once_on_device(once, [] { allow_smem(k_contrast, bytes); });
-        k_contrast<<<nt, DEP_THREADS, bytes, c.stream>>>(p);
-    } else {
-        dep_attrs<T, false>();
-        k_project<T, false><<<nt, DEP_THREADS, dep_smem<T, false, false>(), c.stream>>>(p);
-    }
+    p.G = (float)q;
+    p.c1 = (float)(q - (double)p.G);
+    p.rb_hi = (float)mean;
+    p.rb_lo = (float)(mean - (double)p.rb_hi);
+    static DeviceOnce once;
+    constexpr size_t bytes = dep_smem<float, false, true>();
+    once_on_device(once, [] { allow_smem(k_contrast, bytes); });
+    k_contrast<<<p.ntx * p.nty * ((p.N + p.tz - 1) / p.tz), DEP_THREADS, bytes, c.stream>>>(p);
 }
 
 template <class T>
@@ -2016,7 +2042,6 @@ void launch_check_finite(Ctx &c, const double *d, int64_t n, int *d_flag)
                                            int64_t, int *);                                 \
     template void launch_store_particles<T>(Ctx &, double *, double *, int64_t, int64_t);   \
     template void launch_store_particles_scatter<T>(Ctx &, double *, double *);             \
-    template void launch_density<T>(Ctx &, void *);                                         \
     template void launch_to_f64<T>(Ctx &, const void *, double *, int64_t);                 \
     template void launch_from_f64<T>(Ctx &, const double *, void *, int64_t);               \
     template void launch_check_finite<T>(Ctx &, const double *, int64_t, int *);
