@@ -289,6 +289,33 @@ __global__ void __launch_bounds__(256) k_pk_bin(const typename Cplx<T>::type *d,
         if (sb[i] != 0.0) atomicAdd(&acc[i], sb[i] * inv_n6);
 }
 
+// All three sums of every mode in one launch, for meshes of at most 64: there the launches of the kernels below and the
+// clearing of their histogram cost more than an FP64 square root and two more shared atomics a mode do (32^3 FP64 P(k)
+// 80 us, 87 with them; 64^3 104 and 110).
+template <class T>
+__global__ void __launch_bounds__(256) k_pk_bin_small(const typename Cplx<T>::type *d, int N, int nbins, double inv_n6,
+                                                       double *acc)
+{
+    extern __shared__ double sb[];   // 3 nbins: sums of w |d|^2, w |k|, w
+    for (int i = threadIdx.x; i < 3 * nbins; i += blockDim.x) sb[i] = 0.0;
+    __syncthreads();
+    const int h = N / 2 + 1, e = blockIdx.x * 256 + threadIdx.x, kx = e % h, r = e / h;
+    if (r < N * N) {
+        const int ky = r % N, kz = r / N, ny = ky <= N / 2 ? ky : ky - N, nz = kz <= N / 2 ? kz : kz - N;
+        const int n2 = kx * kx + ny * ny + nz * nz, b = pk_shell(n2);
+        if (b >= 1 && b < nbins) {
+            const typename Cplx<T>::type v = d[e];
+            const double w = (kx > 0 && 2 * kx < N) ? 2.0 : 1.0, re = widen(v.x), im = widen(v.y);
+            atomicAdd(&sb[b], w * (re * re + im * im));
+            atomicAdd(&sb[nbins + b], w * (6.283185307179586476925286766559 * sqrt((double)n2)));
+            atomicAdd(&sb[2 * nbins + b], w);
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < 3 * nbins; i += blockDim.x)
+        if (sb[i] != 0.0) atomicAdd(&acc[i], i < nbins ? sb[i] * inv_n6 : sb[i]);
+}
+
 // hist[n2] = number of modes of the full spectrum with |n|^2 = n2, from the octant 0 <= |n_i| <= N/2 (a block per
 // |n_z|, |n_y|); only shells below nbins are counted
 __global__ void k_pk_modes(int N, int nbins, unsigned int *hist)
@@ -363,6 +390,11 @@ void launch_pk_bin(Ctx &c, const void *spec_in, int nbins, double *d_acc, unsign
     const double inv_n6 = 1.0 / ((double)c.nc * (double)c.nc);
     const int m = c.N / 2;
     cudaMemsetAsync(d_acc, 0, sizeof(double) * 3 * nbins, c.stream);
+    if (c.N <= 64 && nbins <= 2048) {   // 3 nbins doubles of shared memory: 48 KB
+        k_pk_bin_small<T><<<(unsigned)((c.nh + 255) / 256), 256, 3 * sizeof(double) * nbins, c.stream>>>(
+            reinterpret_cast<const typename Cplx<T>::type *>(spec_in), c.N, nbins, inv_n6, d_acc);
+        return;
+    }
     cudaMemsetAsync(hist, 0, sizeof(unsigned int) * (size_t)pk_hist_len(c.N), c.stream);
     const int blocks = std::min((c.N * c.N + 7) / 8, 152 * 8);
     k_pk_bin<T><<<blocks, 256, sizeof(double) * nbins, c.stream>>>(
