@@ -299,6 +299,98 @@ template <class T> __device__ __forceinline__ void acc_merge(Acc<T> &s, const Ac
     s.add(o.hi());
     if constexpr (sizeof(T) == 4) s.c += o.c;
 }
+// Two values side by side.  FP32 takes the packed instructions, one for both values, each rounded as the scalar one's.
+template <class T> struct Pair;
+template <> struct Pair<float> {
+    uint64_t v;
+    static __device__ __forceinline__ Pair of(float a, float b)
+    {
+        Pair r;
+        asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+        return r;
+    }
+    __device__ __forceinline__ float get(int k) const
+    {
+        float a, b;
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+        return k ? b : a;
+    }
+};
+template <> struct Pair<double> {
+    double a, b;
+    static __device__ __forceinline__ Pair of(double a, double b) { return {a, b}; }
+    __device__ __forceinline__ double get(int k) const { return k ? b : a; }
+};
+__device__ __forceinline__ Pair<float> operator+(Pair<float> x, Pair<float> y)
+{
+    Pair<float> r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(x.v), "l"(y.v));
+    return r;
+}
+__device__ __forceinline__ Pair<float> operator-(Pair<float> x, Pair<float> y)
+{
+    Pair<float> r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(x.v), "l"(y.v));
+    return r;
+}
+__device__ __forceinline__ Pair<float> operator*(Pair<float> x, Pair<float> y)
+{
+    Pair<float> r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(x.v), "l"(y.v));
+    return r;
+}
+__device__ __forceinline__ Pair<float> fma(Pair<float> x, Pair<float> y, Pair<float> z)
+{
+    Pair<float> r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(x.v), "l"(y.v), "l"(z.v));
+    return r;
+}
+__device__ __forceinline__ Pair<double> operator+(Pair<double> x, Pair<double> y) { return {x.a + y.a, x.b + y.b}; }
+__device__ __forceinline__ Pair<double> fma(Pair<double> x, Pair<double> y, Pair<double> z)
+{
+    return {::fma(x.a, y.a, z.a), ::fma(x.b, y.b, z.b)};
+}
+// four staged values (FP64: in two parts, 32 records apart)
+__device__ __forceinline__ void pairs(const float4 *v, Pair<float> (&p)[2])
+{
+    const ulonglong2 a = *reinterpret_cast<const ulonglong2 *>(v);
+    p[0].v = a.x;
+    p[1].v = a.y;
+}
+__device__ __forceinline__ void pairs(const double2 *v, Pair<double> (&p)[2])
+{
+    p[0] = {v[0].x, v[0].y};
+    p[1] = {v[32].x, v[32].y};
+}
+
+// Acc of two sums side by side
+template <class T> struct AccPair;
+template <> struct AccPair<double> {
+    Pair<double> s;
+    __device__ __forceinline__ void zero() { s = {0.0, 0.0}; }
+    __device__ __forceinline__ void add_product(Pair<double> a, Pair<double> b) { s = fma(a, b, s); }
+    __device__ __forceinline__ void merge(const double *h, const double *) { s = s + Pair<double>{h[0], h[1]}; }
+    __device__ __forceinline__ Acc<double> get(int k) const { return {s.get(k)}; }
+};
+template <> struct AccPair<float> {
+    Pair<float> s, c;
+    __device__ __forceinline__ void zero() { s = c = Pair<float>::of(0.f, 0.f); }
+    __device__ __forceinline__ void add_two(Pair<float> x, Pair<float> lo)
+    {
+        add(x);
+        c = c + lo;
+    }
+    __device__ __forceinline__ void add(Pair<float> x)
+    {
+        const Pair<float> t = s + x, b = t - s, e = (s - (t - b)) + (x - b);
+        s = t;
+        c = c + e;
+    }
+    __device__ __forceinline__ void add_product(Pair<float> a, Pair<float> b) { add(a * b); }
+    __device__ __forceinline__ void merge(const float *h, const float *l) { add_two(Pair<float>::of(h[0], h[1]), Pair<float>::of(l[0], l[1])); }
+    __device__ __forceinline__ Acc<float> get(int k) const { return {s.get(k), c.get(k)}; }
+};
+
 // Cell, offset and momentum of one particle.
 template <class T> struct PartFU {
     int cell;
@@ -474,18 +566,17 @@ __device__ __forceinline__ void dep_epilogue(const DepParams<T> &p, const T *dn,
     reinterpret_cast<T *>(p.out.p[8])[g] = hb[1] * b[2] + (G4 * s[7] - hc[1] * dc[2]);
 }
 
-// A vertex lane's sums in one plane: of its own row of vertices and of the one at y + 1.
+// A vertex lane's sums in one plane, of its own row of vertices and of the one at y + 1: T00 of both, the others by row.
 template <class T> struct RowSums {
-    Acc<T> t00[2];
-    T q[2][8];
+    AccPair<T> t00;
+    Pair<T> q[2][4];
     __device__ __forceinline__ void zero()
     {
+        t00.zero();
 #pragma unroll
-        for (int i = 0; i < 2; i++) {
-            t00[i].zero();
+        for (int i = 0; i < 2; i++)
 #pragma unroll
-            for (int j = 0; j < 8; j++) q[i][j] = T(0);
-        }
+            for (int j = 0; j < 4; j++) q[i][j] = Pair<T>::of(T(0), T(0));
     }
 };
 
@@ -504,6 +595,15 @@ template <class T, bool FULL, bool DEN> struct DepCol {
     static constexpr int VT = 16 / sizeof(T);              // values in 16 bytes
     static constexpr int W = dep_words<T, FULL>(), R = dep_rec<FULL, DEN>();
     using V = std::conditional_t<sizeof(T) == 4, float4, double2>;
+    // Particles of one cell in a group of 32 from which the warp sums them together, and the row's particles from which
+    // it looks for such cells (a load of one per cell, whose rows it would only slow down, has 32).  A vertex lane takes
+    // 36 products a particle one after another, for two cells: with 16 particles a cell 29 of 32 lanes wait for it.  The
+    // warp takes 3 a particle and some 100 instructions a cell; FP64, where an instruction costs the same for one lane as
+    // for all, four cells at a time.  Deposit at 128^3 without and with it, and of the 8^3 tiles before the columns:
+    // FP32 16 a cell 3.25, 1.94 (1.66), 4 a cell 0.47, 0.49 (0.45), a tenth of the mass in cells of 1000 0.42, 0.26
+    // (0.36); FP64 77.6, 19.9 (33.8), 10.2, 8.2 (7.9), 6.9, 2.8 (5.9) ms.  From 4 or 7 particles on FP32 is slower
+    // (4 a cell 0.78, 0.54), and from 10 on FP64 (16 a cell 28).
+    static constexpr int CROWD = sizeof(T) == 8 ? 4 : 10, CROWDED_ROW = 48;
 
     const DepParams<T> &p;
     V *stage;            // the row's first 32 records in this and the next plane, [par][part][thread]
@@ -554,15 +654,72 @@ template <class T, bool FULL, bool DEN> struct DepCol {
         return r;
     }
     // the row's first 32 records, into part `par` of the stage
-    __device__ __forceinline__ void fetch_row(int par, const DepRow &r)
+    __device__ __forceinline__ void fetch_row(int par, const DepRow &r, int c0 = 0)
     {
-        const int i = threadIdx.x & 31;
+        const int i = c0 + (threadIdx.x & 31);
         if (i < r.total) {
             const V *g = reinterpret_cast<const V *>(p.part + (i < r.nh ? r.sh + i : r.sr + i));
 #pragma unroll
             for (int q = 0; q < PQ; q++) {
                 const unsigned a = (unsigned)__cvta_generic_to_shared(stage + (par * PQ + q) * DEP_THREADS + threadIdx.x);
                 asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(a), "l"(g + q));
+            }
+        }
+    }
+
+    // The sums of records n0 .. n1 - 1 of the staged group, all of one cell, to the cell's 8 corners, into sum
+    // [side][value][line]: a lane forms the T00 sum of a quarter of them for one corner, and two of the other sums of all
+    // of them.
+    __device__ __forceinline__ void crowd_sums(int n0, int n1, T *sum) const
+    {
+        const int lane = threadIdx.x & 31, side = lane & 1, line = (lane >> 1) & 3, part = lane >> 3;
+        const T *wt = rec + (side * (4 / VT) + line / VT) * (32 * VT) + line % VT, *r0 = rec + 32 * (R - 1);
+        Acc<T> t;
+        t.zero();
+#pragma unroll 2
+        for (int n = n0 + part; n < n1; n += 4) {
+            if constexpr (DEN) t.add_two(wt[n * VT], wt[2 * 32 * VT + n * VT]);
+            else t.add_product(wt[n * VT], r0[n]);
+        }
+#pragma unroll
+        for (int k = 8; k < 32; k *= 2) {
+            Acc<T> b;
+            b.s = __shfl_xor_sync(0xffffffffu, t.s, k);
+            if constexpr (sizeof(T) == 4) b.c = __shfl_xor_sync(0xffffffffu, t.c, k);
+            acc_merge(t, b);
+        }
+        T *d = sum + side * (4 * W) + line;
+        if (part == 0) {
+            d[0] = t.hi();
+            if constexpr (sizeof(T) == 4) d[4] = t.lo();
+        }
+        if constexpr (FULL) {
+            const T *q = rec + (8 / VT + 2 * part / VT) * (32 * VT) + 2 * part % VT;
+            Pair<T> qs = Pair<T>::of(T(0), T(0));
+#pragma unroll 4
+            for (int n = n0; n < n1; n++) {
+                const T w = wt[n * VT];
+                qs = fma(Pair<T>::of(w, w), *reinterpret_cast<const Pair<T> *>(q + n * VT), qs);
+            }
+            d[4 * (W - 8 + 2 * part)] = qs.get(0);
+            d[4 * (W - 7 + 2 * part)] = qs.get(1);
+        }
+    }
+    // adds what crowd_sums left for one side of a cell
+    __device__ __forceinline__ void crowd_add(const T *v, RowSums<T> &A, RowSums<T> &B) const
+    {
+#pragma unroll
+        for (int k = 0; k < 2; k++) {
+            RowSums<T> &S = k ? B : A;
+            S.t00.merge(v + 2 * k, v + 4 + 2 * k);
+            if constexpr (FULL) {
+#pragma unroll
+                for (int i = 0; i < 2; i++)
+#pragma unroll
+                    for (int j = 0; j < 4; j++) {
+                        const T *u = v + 4 * (W - 8 + 2 * j) + 2 * k + i;
+                        S.q[i][j] = S.q[i][j] + Pair<T>::of(u[0], u[4]);
+                    }
             }
         }
     }
@@ -590,11 +747,15 @@ template <class T, bool FULL, bool DEN> struct DepCol {
         for_groups(r.total, [&](int c0) {
             const int i = c0 + lane;
             PartFU<T> P{};
+            if (c0 > 0) asm volatile("cp.async.wait_group 0;" ::: "memory");
             int cx = 0;                                // the cell's lower corner in the row's staged potentials
             if (i < r.total) {
-                if (c0 == 0) P = unpack(stage + PAR * PQ * DEP_THREADS + threadIdx.x, DEP_THREADS);
-                else P = unpack(reinterpret_cast<const V *>(p.part + (i < r.nh ? r.sh + i : r.sr + i)), 1);
+                P = unpack(stage + PAR * PQ * DEP_THREADS + threadIdx.x, DEP_THREADS);
                 if (i >= r.nh) cx = P.cell - base;
+            }
+            if (r.total - c0 > 32) {   // the row's next records
+                fetch_row(PAR, r, c0 + 32);
+                asm volatile("cp.async.commit_group;" ::: "memory");
             }
             T wt[8], q00, q[8], ex;
             charges<T, FULL>(p, P, lo + cx, up + cx, wt, q00, q, ex);
@@ -619,47 +780,100 @@ template <class T, bool FULL, bool DEN> struct DepCol {
             auto gather = [&](int n0, int n1, int nm) {
 #pragma unroll(FULL ? 1 : 2)
                 for (int n = n0; n < n1; n++) {
-                    T wn[4], qn[8];
+                    Pair<T> w[2], c[2];
                     const V *v = rv + n + (n < nm ? 32 * (4 / VT) : 0);
-#pragma unroll
-                    for (int k = 0; k < 4 / VT; k++) unpackv(v[32 * k], wn + VT * k);
+                    pairs(v, w);
                     if constexpr (DEN) {
-                        unpackv(v[64], qn);
-                        A.t00[0].add_two(wn[0], qn[0]);
-                        A.t00[1].add_two(wn[1], qn[1]);
-                        B.t00[0].add_two(wn[2], qn[2]);
-                        B.t00[1].add_two(wn[3], qn[3]);
-                        continue;
+                        pairs(v + 64, c);
+                        A.t00.add_two(w[0], c[0]);
+                        B.t00.add_two(w[1], c[1]);
+                    } else {
+                        const T t = r0[n];
+                        A.t00.add_product(w[0], Pair<T>::of(t, t));
+                        B.t00.add_product(w[1], Pair<T>::of(t, t));
                     }
-                    const T t = r0[n];
-                    A.t00[0].add_product(wn[0], t);
-                    A.t00[1].add_product(wn[1], t);
-                    B.t00[0].add_product(wn[2], t);
-                    B.t00[1].add_product(wn[3], t);
                     if constexpr (FULL) {
+                        Pair<T> ww[2][2];
 #pragma unroll
-                        for (int k = 0; k < 8 / VT; k++) unpackv(rv[32 * (8 / VT + k) + n], qn + VT * k);
+                        for (int i = 0; i < 2; i++)
 #pragma unroll
-                        for (int j = 0; j < 8; j++) {
-                            A.q[0][j] += wn[0] * qn[j];
-                            A.q[1][j] += wn[1] * qn[j];
-                            B.q[0][j] += wn[2] * qn[j];
-                            B.q[1][j] += wn[3] * qn[j];
+                            for (int k = 0; k < 2; k++) ww[k][i] = Pair<T>::of(w[k].get(i), w[k].get(i));
+#pragma unroll
+                        for (int h = 0; h < 2; h++) {
+                            pairs(rv + 32 * (8 / VT + h * 4 / VT) + n, c);
+#pragma unroll
+                            for (int j = 0; j < 2; j++)
+#pragma unroll
+                                for (int i = 0; i < 2; i++) {
+                                    A.q[i][2 * h + j] = fma(ww[0][i], c[j], A.q[i][2 * h + j]);
+                                    B.q[i][2 * h + j] = fma(ww[1][i], c[j], B.q[i][2 * h + j]);
+                                }
                         }
                     }
                 }
             };
-            gather(max(r.prev - c0, 0), min(r.end - c0, 32), r.mid - c0);
-            if (p.cyclic) gather(max(r.wrap - c0, 0), min(r.total - c0, 32), 32);   // lane 0: the row's last cell
+            int g0 = r.prev, g1 = r.end, g2 = r.wrap;
+            if (r.total >= CROWDED_ROW) {   // cells with many particles in this group: by the whole warp
+                const int own0 = max(r.mid - c0, 0), own1 = min(r.end - c0, 32);
+                unsigned m = __ballot_sync(0xffffffffu, own1 - own0 >= CROWD);
+                const int n1 = min(r.nh - c0, 32);
+                const bool front = n1 >= CROWD;   // the cell x0 - 1
+                if (lane == 0 ? front : (m >> (lane - 1)) & 1) g0 = r.mid;
+                if ((m >> lane) & 1) g1 = r.mid;
+                if ((m >> (nx - 1)) & 1) g2 = r.total;
+                T *sum = xch + (PAR * DROWS + w) * (32 * W);   // this row's part of the exchange, free until the barrier
+                if constexpr (sizeof(T) == 8) {   // four cells at a time, the cell x0 - 1 among the first
+                    int f = 0;
+                    if (front) crowd_sums(0, n1, sum + 8 * W * f++);
+                    while (f || m) {
+                        unsigned now = m;
+                        for (int k = f; m && k < 4; k++) {
+                            const int o = __ffs(m) - 1;
+                            m &= m - 1;
+                            crowd_sums(__shfl_sync(0xffffffffu, own0, o), __shfl_sync(0xffffffffu, own1, o), sum + 8 * W * k);
+                        }
+                        now &= ~m;
+                        __syncwarp();
+                        // where this vertex's shares of its own cell and of the one at x - 1 are
+                        auto slot = [&](int o) { return (now >> o) & 1 ? f + __popc(now & ((1u << o) - 1)) : -1; };
+                        const int own = slot(lane);
+                        int prev = lane > 0 ? slot(lane - 1) : f ? 0 : p.cyclic ? slot(nx - 1) : -1;
+                        if (lane >= nx) prev = -1;
+                        if (own >= 0 || prev >= 0) crowd_add(own >= 0 ? sum + 8 * W * own : sum + 8 * W * prev + 4 * W, A, B);
+                        if (own >= 0 && prev >= 0) crowd_add(sum + 8 * W * prev + 4 * W, A, B);
+                        __syncwarp();
+                        f = 0;
+                    }
+                } else if (front || m) {   // one at a time: fewer registers
+                    int o = -1, e0 = 0, e1 = n1;
+                    while (true) {
+                        if (o >= 0 || front) {
+                            crowd_sums(e0, e1, sum);
+                            __syncwarp();
+                            const int next = p.cyclic && o == nx - 1 ? 0 : o + 1;
+                            if (lane == o || (lane == next && lane < nx)) crowd_add(sum + (lane == o ? 0 : 4 * W), A, B);
+                            __syncwarp();
+                        }
+                        if (!m) break;
+                        o = __ffs(m) - 1;
+                        m &= m - 1;
+                        e0 = __shfl_sync(0xffffffffu, own0, o);
+                        e1 = __shfl_sync(0xffffffffu, own1, o);
+                    }
+                }
+            }
+            gather(max(g0 - c0, 0), min(g1 - c0, 32), r.mid - c0);
+            if (p.cyclic) gather(max(g2 - c0, 0), min(r.total - c0, 32), 32);   // lane 0: the row's last cell
             __syncwarp();
         });
         T *xo = xch + (PAR * DROWS + w) * (32 * W) + lane;
         if (iz >= 0) {   // the sums for the row at y + 1
-            xo[0] = A.t00[1].hi();
-            if constexpr (sizeof(T) == 4) xo[32] = A.t00[1].lo();
+            const Acc<T> t = A.t00.get(1);
+            xo[0] = t.hi();
+            if constexpr (sizeof(T) == 4) xo[32] = t.lo();
             if constexpr (FULL) {
 #pragma unroll
-                for (int j = 0; j < 8; j++) xo[(W - 8 + j) * 32] = A.q[1][j];
+                for (int j = 0; j < 8; j++) xo[(W - 8 + j) * 32] = A.q[1][j / 2].get(j & 1);
             }
         }
         asm volatile("cp.async.wait_group 1;" ::: "memory");   // the potentials of plane z + 2
@@ -670,7 +884,7 @@ template <class T, bool FULL, bool DEN> struct DepCol {
         rn = range(nb);
         if (out) {
             const T *xi = xo - 32 * W;
-            Acc<T> S = A.t00[0], S2;
+            Acc<T> S = A.t00.get(0), S2;
             S2.s = xi[0];
             if constexpr (sizeof(T) == 4) S2.c = xi[32];
             acc_merge(S, S2);
@@ -688,7 +902,7 @@ template <class T, bool FULL, bool DEN> struct DepCol {
             } else {
                 T s[8];
 #pragma unroll
-                for (int j = 0; j < 8; j++) s[j] = A.q[0][j] + xi[(W - 8 + j) * 32];
+                for (int j = 0; j < 8; j++) s[j] = A.q[0][j / 2].get(j & 1) + xi[(W - 8 + j) * 32];
                 dep_epilogue(p, ring + slot(DRING - 1) * DPN + col, ring + sc * DPN + col, ring + slot(1) * DPN + col, f2, dS,
                              s, g, k0);
             }

@@ -43,3 +43,30 @@ def test_fp64_power_of_clumps(pm):  # noqa: F811
     """A tenth of the mass in cells of 10^4: 1.3 times the even load (10 times in the deposit's columns)."""
     t = [power_ms(make(pm, pm.PM_FP64, pm.PM_NEWTONIAN, clump=c)) for c in (0, 10000)]
     assert t[1] < 3 * t[0], t
+
+
+def stage_ms(s, stage):
+    for _ in range(2):
+        s.step()
+    s.timings()
+    for _ in range(5):
+        s.step()
+    ms = s.timings()[0][stage]
+    s.close()
+    return ms
+
+
+# a particle of a dense load (or of one with clumps) against one of an even load of one a cell
+@pytest.mark.parametrize("precision,bound", [("PM_MIXED", 1.2), ("PM_FP64", 1.5)])
+def test_deposit_of_a_dense_load(pm, precision, bound):  # noqa: F811
+    """16 particles a cell cost 0.8 (FP32) and 0.6 (FP64) of the even load's time a particle; 1.5 and 2.3 where the
+    vertex lanes sum them one by one."""
+    t = [stage_ms(make(pm, getattr(pm, precision), 0, c), "project") / c for c in (1, 16)]
+    assert t[1] < bound * t[0], t
+
+
+@pytest.mark.parametrize("precision,bound", [("PM_MIXED", 3.0), ("PM_FP64", 2.0)])
+def test_deposit_of_clumps(pm, precision, bound):  # noqa: F811
+    """A tenth of the mass in cells of 1000: 2 (FP32) and 1.2 (FP64) times the even load; 4 and 3.3 before."""
+    t = [stage_ms(make(pm, getattr(pm, precision), 0, 1.0, c), "project") for c in (0, 1000)]
+    assert t[1] < bound * t[0], t
