@@ -1184,20 +1184,70 @@ __device__ __forceinline__ bool carry_cells(double v, int N, double &f, int &car
 }
 __device__ __forceinline__ bool carry_cells(float, int, float &, int &) { return false; }
 
+// FP64: the particles of the rows of cells of a plane.  An FP64 instruction takes the pipe as long for one lane as for
+// 32, so where a row has more than 32 particles, or all rows so few that most lanes would be idle, the warps share all
+// rows' particles in groups of 32 (128^3, own rows and shared ones: z = 1 1.89 -> 1.46 ms, half a particle a cell 1.21 ->
+// 0.72, 0.05 0.98 -> 0.36, a tenth of the mass in cells of 1000 2.39 -> 1.44).  From 192 particles a plane on, 6 of 8
+// full groups, there is nothing to gain.  FP32 kernels keep their own rows: with the table they were slower at one
+// particle a cell (256^3 0.46 -> 0.52 ms), which the rows of more than 32 do not make up for (z = 1 0.70 -> 0.71).
+struct alignas(16) KickRows {
+    int end[KROWS];   // particles of the rows up to this one
+    int off[KROWS];   // particle j of all rows' is off[its row] + j
+    int shared;       // the warps share them
+
+    // by a whole warp, whose lane l < KROWS has row l's particles s .. e - 1
+    __device__ __forceinline__ void set(int s, int e)
+    {
+        const int lane = threadIdx.x & 31, n = lane < KROWS ? e - s : 0;
+        int sum = n;
+#pragma unroll
+        for (int o = 1; o < KROWS; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, sum, o);
+            if (lane >= o) sum += v;
+        }
+        const bool full = __any_sync(0xffffffffu, n > 32);
+        if (lane < KROWS) {
+            end[lane] = sum;
+            off[lane] = e - sum;
+        }
+        if (lane == KROWS - 1) shared = full || sum <= 24 * KROWS;
+    }
+    // particle j of all rows' and its row; i = -1: none
+    __device__ __forceinline__ void find(unsigned j, int &i, int &r) const
+    {
+        const int4 a = *reinterpret_cast<const int4 *>(end), b = *reinterpret_cast<const int4 *>(end + 4);
+        r = (j >= (unsigned)a.x) + (j >= (unsigned)a.y) + (j >= (unsigned)a.z) + (j >= (unsigned)a.w) +
+            (j >= (unsigned)b.x) + (j >= (unsigned)b.y) + (j >= (unsigned)b.z);
+        i = j < (unsigned)b.w ? off[r] + (int)j : -1;
+    }
+    // a lane's first particle: `group` 32 of all rows' where they are shared
+    __device__ __forceinline__ void first(int w, int group, int &i, int &r) const
+    {
+        if (shared) {
+            find(32 * group + (threadIdx.x & 31), i, r);
+        } else {
+            const int j = (w > 0 ? end[w - 1] : 0) + (threadIdx.x & 31);
+            r = w;
+            i = j < end[w] ? off[w] + j : -1;
+        }
+    }
+};
+static_assert(KROWS == 8, "find() compares with 7 ends");
+
 // CORR: with the force correction of a Newtonian context
 template <class T, bool NEWT, bool CORR = false>
 __device__ __forceinline__ void kick_tile(const KdParams<T> &p, const int b)
 {
     extern __shared__ __align__(16) unsigned char smem[];
+    constexpr bool FP64 = sizeof(T) == 8;
     constexpr int PQ = sizeof(Particle<T>) / 16;
-    using V = std::conditional_t<sizeof(T) == 4, float4, double2>;
+    using V = std::conditional_t<FP64, double2, float4>;
     T *ring = reinterpret_cast<T *>(smem);
     Vtx4<T> *sv = reinterpret_cast<Vtx4<T> *>(ring);                           // [KRING][KPN]
     T *sb = NEWT ? ring : ring + 4 * KRING * KPN;                              // B_z (Newtonian: phi) [KRING][KPN]
     const int N = p.N, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int x0 = (b % p.ntx) * p.nrow, y0 = ((b / p.ntx) % (N / KROWS)) * KROWS, z0 = b / (p.ntx * (N / KROWS)) * p.tz;
     const int nx = min(p.nrow, N - x0), nz = min(p.tz, N - z0);
-    const int row = (y0 + w) * N + x0;
 
     // this thread's vertices of a plane: where they come from (-1: none)
     int go[KLD];
@@ -1233,51 +1283,69 @@ __device__ __forceinline__ void kick_tile(const KdParams<T> &p, const int b)
                 sb[slot * KPN + tid + q * KD_THREADS] = vb[q];
             }
     };
-    // a row's first 32 records, ahead of their plane
-    V nxt[PQ];
-    auto fetch = [&](int s, int e) {
-        if (lane < e - s) {   // not s + lane < e: that sum can pass 2^31 - 1
-#pragma unroll
-            for (int q = 0; q < PQ; q++) nxt[q] = reinterpret_cast<const V *>(p.part + s + lane)[q];
-        }
-    };
     for (int i = 0; i < 4; i++) {   // planes z0 - 1 .. z0 + 2
         load(z0 - 1 + i);
         keep(i);
     }
-    const int32_t *st = p.start + z0 * (N * N) + row;
-    int s0 = __ldg(st), e0 = __ldg(st + nx), s1 = 0, e1 = 0;
-    if (nz > 1) {
-        s1 = __ldg(st + N * N);
-        e1 = __ldg(st + N * N + nx);
+    const int32_t *st = p.start + z0 * (N * N) + y0 * N + x0;
+    __shared__ KickRows rows[FP64 ? 4 : 1];   // FP64 only
+    // this lane's first particle of a plane, fetched a plane ahead
+    V nxt[PQ];
+    auto fetch = [&](int i) {
+#pragma unroll
+        for (int q = 0; q < PQ; q++) nxt[q] = reinterpret_cast<const V *>(p.part + i)[q];
+    };
+    int i0 = -1, r0 = w;                  // FP64: that particle and its row
+    int s0 = 0, e0 = 0, s1 = 0, e1 = 0;   // FP32: this warp's row in this plane and the next
+    if constexpr (FP64) {   // the rows of a plane are counted two planes ahead, by a warp after the other
+        const int32_t *q = st + w * (N * N) + (lane % KROWS) * N;
+        if (w < 2 && w < nz) rows[w].set(__ldg(q), __ldg(q + nx));
+        __syncthreads();
+        rows[0].first(w, (w + z0) % KROWS, i0, r0);
+        if (i0 >= 0) fetch(i0);
+    } else {
+        const int32_t *q = st + w * N;
+        s0 = __ldg(q);
+        e0 = __ldg(q + nx);
+        if (nz > 1) {
+            s1 = __ldg(q + N * N);
+            e1 = __ldg(q + N * N + nx);
+        }
+        if (lane < e0 - s0) fetch(s0 + lane);
+        __syncthreads();
     }
-    fetch(s0, e0);
-    __syncthreads();
 
     int sc = 0;   // slot of plane z - 1
     for (int iz = 0; iz < nz; iz++) {
         const int z = z0 + iz;
         if (iz + 1 < nz) load(z + 3);
+        const bool ahead = iz + 2 < nz && (!FP64 || w == iz % KROWS);
         int s2 = 0, e2 = 0;
-        if (iz + 2 < nz) {
-            s2 = __ldg(st + (iz + 2) * (N * N));
-            e2 = __ldg(st + (iz + 2) * (N * N) + nx);
+        if (ahead) {
+            const int32_t *q = st + (iz + 2) * (N * N) + (FP64 ? lane % KROWS : w) * N;
+            s2 = __ldg(q);
+            e2 = __ldg(q + nx);
         }
         V rec[PQ];
 #pragma unroll
         for (int q = 0; q < PQ; q++) rec[q] = nxt[q];
-        fetch(s1, e1);
-        const int base = z * (N * N) + row;
-        for_groups(e0 - s0, [&](int c0) {
-            if (c0 + lane >= e0 - s0) return;
-            const int i = s0 + c0 + lane;
-            if (c0 > 0) {
+        int i = i0, r = r0;
+        if constexpr (FP64) {
+            i0 = -1;
+            if (iz + 1 < nz) rows[(iz + 1) % 4].first(w, (w + z + 1) % KROWS, i0, r0);
+            if (i0 >= 0) fetch(i0);
+        } else {
+            if (lane < e1 - s1) fetch(s1 + lane);
+        }
+        auto record = [&](int i) {
 #pragma unroll
-                for (int q = 0; q < PQ; q++) rec[q] = reinterpret_cast<const V *>(p.part + i)[q];
-            }
+            for (int q = 0; q < PQ; q++) rec[q] = reinterpret_cast<const V *>(p.part + i)[q];
+        };
+        // particle i, in row r
+        auto move = [&](int i, int r) {
             Particle<T> P = *reinterpret_cast<const Particle<T> *>(rec);
-            const int cx = P.cell - base;
-            const int vo = w * KPX + cx;   // vertex at stencil offset (0, 0) in its plane
+            const int cx = P.cell - (z * (N * N) + (y0 + r) * N + x0);
+            const int vo = r * KPX + cx;   // vertex at stencil offset (0, 0) in its plane
             const T fx = P.f[0], fy = P.f[1], fz = P.f[2];
             T u[3] = {P.u[0], P.u[1], P.u[2]};
             T dx[3];
@@ -1285,7 +1353,7 @@ __device__ __forceinline__ void kick_tile(const KdParams<T> &p, const int b)
 #pragma unroll
             for (int k = 0; k < 4; k++) slot[k] = (sc + k >= KRING ? sc + k - KRING : sc + k) * KPN + vo;
             const T *const pb[4] = {sb + slot[0], sb + slot[1], sb + slot[2], sb + slot[3]};
-            if constexpr (CORR) add_correction(p, x0 + cx, y0 + w, z, fx, fy, fz, u);
+            if constexpr (CORR) add_correction(p, x0 + cx, y0 + r, z, fx, fy, fz, u);
             if constexpr (NEWT) {
                 const T hn = p.halfN;
                 const T Wx[4] = {0, T(1) - fx, fx, 0}, Wy[4] = {0, T(1) - fy, fy, 0}, Wz[4] = {0, T(1) - fz, fz, 0};
@@ -1318,7 +1386,7 @@ __device__ __forceinline__ void kick_tile(const KdParams<T> &p, const int b)
                 for (int d = 0; d < 3; d++) dx[d] = p.dt_drift_N * (u[d] * fac + val[2 + d]);
             }
             const T fo[3] = {fx, fy, fz};
-            const int io[3] = {x0 + cx, y0 + w, z};
+            const int io[3] = {x0 + cx, y0 + r, z};
             int inew[3];
             bool near = sizeof(T) == 8;
             if constexpr (sizeof(T) == 8) {
@@ -1350,15 +1418,33 @@ __device__ __forceinline__ void kick_tile(const KdParams<T> &p, const int b)
             P.cell = (inew[2] * N + inew[1]) * N + inew[0];
             p.part[i] = P;
             atomicAdd(&p.count[P.cell], 1);
-        });
+        };
+        if constexpr (FP64) {
+            const KickRows &now = rows[iz % 4];
+            for (unsigned c = 32 * ((unsigned)(w + z) % KROWS);;) {
+                if (i >= 0) move(i, r);
+                if (!now.shared || (c += 32 * KROWS) >= (unsigned)now.end[KROWS - 1]) break;
+                now.find(c + lane, i, r);
+                if (i >= 0) record(i);
+            }
+            if (ahead) rows[(iz + 2) % 4].set(s2, e2);
+        } else {
+            // (unsigned: a particle number plus 32 can pass 2^31 - 1)
+            for (unsigned k = (unsigned)s0 + lane; k < (unsigned)e0; k += 32) {
+                if (k >= (unsigned)s0 + 32) record(k);
+                move(k, w);
+            }
+        }
         // plane z + 3 into the slot of plane z - 2, last read before the barrier of the plane before
         if (iz + 1 < nz) keep(sc + 4 >= KRING ? sc + 4 - KRING : sc + 4);
         __syncthreads();
+        if constexpr (!FP64) {
+            s0 = s1;
+            e0 = e1;
+            s1 = s2;
+            e1 = e2;
+        }
         sc = sc + 1 == KRING ? 0 : sc + 1;
-        s0 = s1;
-        e0 = e1;
-        s1 = s2;
-        e1 = e2;
     }
 }
 

@@ -70,3 +70,10 @@ def test_deposit_of_clumps(pm, precision, bound):  # noqa: F811
     """A tenth of the mass in cells of 1000: 2 (FP32) and 1.2 (FP64) times the even load; 4 and 3.3 before."""
     t = [stage_ms(make(pm, getattr(pm, precision), 0, 1.0, c), "project") for c in (0, 1000)]
     assert t[1] < bound * t[0], t
+
+
+def test_fp64_kick_of_sparse_and_crowded_rows(pm):  # noqa: F811
+    """0.05 particles a cell 0.3 and a tenth of the mass in cells of 1000 1.2 times the even load; 0.8 and 2 where each
+    warp takes its own row."""
+    t = [stage_ms(make(pm, pm.PM_FP64, 0, *load), "kick_drift") for load in ((1.0,), (0.05,), (1.0, 1000))]
+    assert t[1] < 0.55 * t[0] and t[2] < 1.6 * t[0], t
