@@ -148,16 +148,19 @@ __device__ __forceinline__ T hc_remainder(T ph, const T (&up)[3], const T (&dn)[
 // (z - 1, y), (z - 1, y - 1), cells x - 1 then x.  This order is kept: the force correction feeds R through BF16
 // layers, where a change in the last bit of R changes the momenta by 1e-3 of their size, so a faster summation
 // order (the columns below need 0.33 ms at 288^3 with 201^3 particles) is not taken here.
-// What bounds it: instruction issue of the 8 dependent sums per vertex.  256^3 with a particle per cell 0.51 ->
-// 0.35 ms, 288^3 with 201^3 particles at z = 2 0.65 -> 0.57, against the general tile kernel that staged whole charge
-// records and searched each particle's cell.
+// What bounds it: instruction issue of the 8 dependent sums per vertex.  Staging: in an even tile each thread takes
+// the particles of its two cells, else every 512th particle, whose row it finds by halving the 81 rows' offsets (a
+// row's cells follow each other in memory).  256^3 at z = 50 0.37 ms with the search alone, 0.35 with both; with its
+// own cells alone, and the warp for full ones, z = 1 0.65 and 128^3 with 16 a cell 2.0, with both 0.57 and 0.71.
+// The general tile kernel before it, which staged whole charge records, took 0.52 ms at 256^3, z = 50.
 // ---------------------------------------------------------------------------
 constexpr int MT = 8, MR = MT + 1, MCELLS = MR * MR * MR, MTHREADS = MT * MT * MT;
-constexpr int MOWN = 8;     // particles of two cells that their thread stages itself
+constexpr int MEVEN = 5;    // particles of two cells up to which a thread stages those of its own
 
 template <class I> struct MassSmem {
     float4 rec[MCAP];                         // f
     I off[MCELLS + 1];                        // exclusive scan of the cells' counts
+    I base[2][MR * MR];                       // particle j of the tile is base[..][its row] + j: [0] for a row's first cell
     I warp[MTHREADS / 32];
 };
 
@@ -197,35 +200,35 @@ template <class I> __device__ __forceinline__ void mass_tile(const DepParams<flo
     const I e = before + inc - n[0] - n[1];
     if (2 * tid <= MCELLS) sm.off[2 * tid] = e;
     if (2 * tid + 1 <= MCELLS) sm.off[2 * tid + 1] = e + n[0];
-    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 2; q++) {   // the row's cells after its first one follow each other in memory, too
+        const int i = 2 * tid + q;
+        if (i < MCELLS && i % MR < 2) sm.base[i % MR][i / MR] = s[q] - (q ? e + n[0] : e);
+    }
+    const bool even = !__syncthreads_or(n[0] + n[1] > MEVEN) && total <= MCAP;
 
     const int ox = tid % MT, oy = (tid / MT) % MT, oz = tid / (MT * MT);
     Acc<float> acc;
     acc.zero();
     for (I lo = 0; lo < total; lo += MCAP) {
         const I hi = min(total, lo + MCAP);
-        // each thread stages the particles of its two cells, MOWN at most; the warp
-        // together stages what is left in crowded cells
-        auto stage = [&](int first0, int n0, int first1, int k, int to) {
-            const float *q = reinterpret_cast<const float *>(p.part + (k < n0 ? first0 + k : first1 + (k - n0)));
+        auto stage = [&](I i, int to) {
+            const float *q = reinterpret_cast<const float *>(p.part + i);
             const float2 xy = __ldg(reinterpret_cast<const float2 *>(q + 2));
             sm.rec[to] = make_float4(xy.x, xy.y, __ldg(q + 4), 0.f);
         };
-        // its share k0 .. k1 - 1 of the pair's particles (at most n_part, so that an int holds k but not k + 32)
-        const I m = (I)n[0] + n[1];
-        const int k0 = (int)min(max(lo - e, I(0)), m), k1 = (int)max(min(m, hi - e), I(0));
-        const int ko = k0 + min(max(k1 - k0, 0), MOWN);
+        if (even) {   // a thread those of its two cells
 #pragma unroll 1
-        for (int k = k0; k < ko; k++) stage(s[0], n[0], s[1], k, (int)(e - lo) + k);
-        for (unsigned left = __ballot_sync(0xffffffffu, ko < k1); left; left &= left - 1) {
-            const int o = __ffs(left) - 1;
-            const int f0 = __shfl_sync(0xffffffffu, s[0], o), m0 = __shfl_sync(0xffffffffu, n[0], o),
-                      f1 = __shfl_sync(0xffffffffu, s[1], o), to = (int)(__shfl_sync(0xffffffffu, e, o) - lo),
-                      k = __shfl_sync(0xffffffffu, ko, o), end = __shfl_sync(0xffffffffu, k1, o);
-            for_groups(end - k, [&](int c) {
-                if (c + lane < end - k) stage(f0, m0, f1, k + c + lane, to + k + c + lane);
-            });
-        }
+            for (int k = 0; k < n[0] + n[1]; k++) stage(k < n[0] ? s[0] + k : s[1] + (k - n[0]), (int)e + k);
+        } else        // a thread every 512th, its row by halving
+            for (int k = tid; k < (int)(hi - lo); k += MTHREADS) {
+                const I j = lo + k;
+                int row = 0;
+#pragma unroll
+                for (int half = 64; half > 0; half >>= 1)
+                    if (row + half < MR * MR && sm.off[MR * (row + half)] <= j) row += half;
+                stage(sm.base[j >= sm.off[MR * row + 1]][row] + j, k);
+            }
         __syncthreads();
         // vertex o receives from cells o - d, d in {0,1}^3, weight (d ? f : 1 - f) per axis; the x-neighbours
         // (region x = ox and ox + 1) are adjacent in the particle order

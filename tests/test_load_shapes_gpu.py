@@ -77,3 +77,10 @@ def test_fp64_kick_of_sparse_and_crowded_rows(pm):  # noqa: F811
     warp takes its own row."""
     t = [stage_ms(make(pm, pm.PM_FP64, 0, *load), "kick_drift") for load in ((1.0,), (0.05,), (1.0, 1000))]
     assert t[1] < 0.55 * t[0] and t[2] < 1.6 * t[0], t
+
+
+def test_mass_deposit_of_a_dense_load(pm):  # noqa: F811
+    """16 particles a cell cost 0.6 of the even load's time a particle in the mixed Newtonian deposit; 1.7 where a warp
+    stages full cells one after another."""
+    t = [stage_ms(make(pm, pm.PM_MIXED, pm.PM_NEWTONIAN, c), "project") / c for c in (1, 16)]
+    assert t[1] < 1.1 * t[0], t
