@@ -311,7 +311,9 @@ pm_status pm_fft_shapes(pm_ctx *ctx, int32_t force_y, int32_t force_z, int32_t *
  * is half of it, which spreads a small or unevenly loaded mesh over more
  * CTAs.  Both shapes
  * compute the same sums (only the order of additions inside a cell may
- * differ).  force 0 or 1 selects a shape; -2 keeps the current one; -1 times
+ * differ).  The deposit of mixed Newtonian contexts has one shape: there the
+ * choice is kept and reported, changes nothing, and -1 keeps shape 0 without
+ * timing.  force 0 or 1 selects a shape; -2 keeps the current one; -1 times
  * the deposit of the context's current state with both shapes and keeps the
  * faster one (the context must hold particles and be between steps; the
  * trial deposits write into internal scratch, so the fields pm_get_field
@@ -379,10 +381,10 @@ pm_status pm_ensemble_set_batched(pm_ensemble *e, int32_t batched);
 /* Current stream count and batched flag (either pointer may be NULL). */
 pm_status pm_ensemble_get_mode(pm_ensemble *e, int32_t *n_streams, int32_t *batched);
 
-/* Autotuner: first the FFT column-pass shapes and the projection's bin shape
- * of every distinct mesh size and precision (pm_fft_shapes and
- * pm_deposit_shape with -1 on the first box of that size, the choice copied
- * to the others; no box advances), then for each candidate number of streams
+/* Autotuner: first the FFT column-pass shapes of every distinct mesh size and
+ * precision and the projection's shape of every distinct mesh size, precision
+ * and mode (pm_fft_shapes and pm_deposit_shape with -1 on the first such box,
+ * the choice copied to the others; no box advances), then for each candidate number of streams
  * (1, 2, 4, 8, at most nbox), per-box and batched, one untimed and two timed
  * graph-captured ensemble steps, keeping the fastest; *n_streams receives the
  * stream count (pm_ensemble_get_mode reports the batched flag).  Each trial

@@ -1153,7 +1153,8 @@ pm_status pm_deposit_shape(pm_ctx *ctx, int32_t force, int32_t *shape)
         if (!c.have_particles || c.stage != 0 || c.step >= c.cfg.n_steps)
             return fail(c, PM_ERR_STATE, "pm_deposit_shape: timing needs particles between steps");
         const StepScalars s = scalars(c, c.step, false);
-        if (c.mixed) tune_deposit_shape<float>(c, s);
+        if (c.mixed && c.newtonian) c.dep_shape = 0;   // k_mass has one shape: nothing to choose
+        else if (c.mixed) tune_deposit_shape<float>(c, s);
         else tune_deposit_shape<double>(c, s);
         cudaError_t e = c.stream ? cudaStreamSynchronize(c.stream) : cudaDeviceSynchronize();
         if (e == cudaSuccess) e = cudaGetLastError();

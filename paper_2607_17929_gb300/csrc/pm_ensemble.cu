@@ -349,12 +349,13 @@ pm_status pm_ensemble_tune(pm_ensemble *e, int32_t *n_streams)
                                                   e->box[first]->c.col_shape[1], nullptr, nullptr);
         if (st != PM_OK) return st;
     }
-    // deposit chunk capacity, once per distinct mesh size and precision (between steps, so side-effect free)
+    // deposit column length, once per distinct mesh size, precision and mode (the mixed Newtonian deposit has no choice;
+    // between steps, so side-effect free)
     for (size_t b = 0; b < e->box.size(); b++) {
         pm::Ctx &c = e->box[b]->c;
         size_t first = b;
         for (size_t a = 0; a < b; a++)
-            if (e->box[a]->c.N == c.N && e->box[a]->c.mixed == c.mixed) {
+            if (e->box[a]->c.N == c.N && e->box[a]->c.mixed == c.mixed && e->box[a]->c.newtonian == c.newtonian) {
                 first = a;
                 break;
             }

@@ -2172,7 +2172,7 @@ void launch_kick_batch(Ctx *const *cs, const StepScalars *ss, int n, bool full, 
     }
 }
 
-// Time the deposit of the context's current state with each chunk capacity and keep the fastest.  The trial
+// Time the deposit of the context's current state with each column length and keep the fastest.  The trial
 // deposits write into the spectrum buffer, which holds nothing between steps (9 half spectra hold more than
 // 9 real fields), so the sources the caller can read stay as they were; the k = 0 slots they also add to are
 // cleared again.
@@ -2304,7 +2304,7 @@ template <> void launch_density<float>(Ctx &c, void *real_out)
     p.N = c.N;
     p.newtonian = 1;
     p.mass = 1.f;
-    dep_tiles(p, false, c.dep_shape);
+    dep_tiles(p, false, 0);
     const double mean = (double)c.np / (double)c.nc, q = (double)c.nc / (double)c.np;
     p.G = (float)q;
     p.c1 = (float)(q - (double)p.G);

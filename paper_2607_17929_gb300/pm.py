@@ -324,8 +324,8 @@ def pm_io_wait(ctx):
 
 
 def pm_deposit_shape(ctx, force=-1):
-    """Select (0, 1), keep (-2) or, with -1, time and keep the faster projection bin shape; returns the shape
-    in use."""
+    """Select (0, 1), keep (-2) or, with -1, time and keep the faster column length of the projection; returns the
+    shape in use (mixed Newtonian contexts have one: -1 keeps 0 without timing)."""
     v = C.c_int32()
     _check(ctx, lib.pm_deposit_shape(ctx, int(force), C.byref(v)))
     return v.value
