@@ -72,15 +72,6 @@ struct Background {
     }
 };
 
-bool valid_n(int n)
-{
-    if (n < 8 || n > 1024 || n % 8) return false;
-    int m = n;
-    while (m % 2 == 0) m /= 2;
-    while (m % 3 == 0) m /= 3;
-    return m == 1;
-}
-
 pm_status fail(Ctx &c, pm_status st, const std::string &msg)
 {
     c.err = msg;
@@ -655,7 +646,7 @@ pm_status pm_init(const pm_config *cfg, pm_ctx **out)
 {
     if (!cfg || !out) return PM_ERR_INVALID_ARG;
     *out = nullptr;
-    if (!valid_n(cfg->n_mesh)) return PM_ERR_UNSUPPORTED_SIZE;
+    if (!is_mesh_size(cfg->n_mesh)) return PM_ERR_UNSUPPORTED_SIZE;
     if (cfg->n_steps < 1 || cfg->n_part < 1 || cfg->n_part >= (int64_t)1 << 31 || !(cfg->box_mpch > 0) ||
         !(cfg->omega_m > 0 && cfg->omega_m <= 1) || !(cfg->z_init > cfg->z_final) || !(cfg->z_final > -1) ||
         (cfg->precision != PM_FP64 && cfg->precision != PM_MIXED) || (cfg->flags & ~(PM_NEWTONIAN | PM_FULL_HC | PM_B_SPACESPACE)))

@@ -256,36 +256,6 @@ template <class T, int N> struct FastPasses {
     }
 };
 
-// calls f.template operator()<N>() for the mesh size n; false for any other number
-template <class F> bool with_fast_n(int n, F &&f)
-{
-    switch (n) {
-    case 8: f.template operator()<8>(); return true;
-    case 16: f.template operator()<16>(); return true;
-    case 24: f.template operator()<24>(); return true;
-    case 32: f.template operator()<32>(); return true;
-    case 48: f.template operator()<48>(); return true;
-    case 64: f.template operator()<64>(); return true;
-    case 72: f.template operator()<72>(); return true;
-    case 96: f.template operator()<96>(); return true;
-    case 128: f.template operator()<128>(); return true;
-    case 144: f.template operator()<144>(); return true;
-    case 192: f.template operator()<192>(); return true;
-    case 216: f.template operator()<216>(); return true;
-    case 256: f.template operator()<256>(); return true;
-    case 288: f.template operator()<288>(); return true;
-    case 384: f.template operator()<384>(); return true;
-    case 432: f.template operator()<432>(); return true;
-    case 512: f.template operator()<512>(); return true;
-    case 576: f.template operator()<576>(); return true;
-    case 648: f.template operator()<648>(); return true;
-    case 768: f.template operator()<768>(); return true;
-    case 864: f.template operator()<864>(); return true;
-    case 1024: f.template operator()<1024>(); return true;
-    default: return false;
-    }
-}
-
 }  // namespace
 
 template <class T>
@@ -307,7 +277,7 @@ void fft_forward(Ctx &c, int nf, const void *const *real_in, void *const *spec_o
         F::template cols<true>(c, nf, po, -1);
         c.mark(EV_FWD_Z);
     };
-    with_fast_n(N, fast);
+    with_mesh_size(N, fast);
 }
 
 template <class T>
@@ -329,14 +299,14 @@ void fft_inverse(Ctx &c, int nf, void *const *spec_in, void *const *real_out)
         F::rows(c, nf, pi, po, +1);
         c.mark(EV_INV_X);
     };
-    with_fast_n(N, fast);
+    with_mesh_size(N, fast);
 }
 
 template <class T>
 bool fft_shapes_tunable(const Ctx &c)
 {
     bool t = false;
-    with_fast_n(c.N, [&]<int NN>() { t = Lines<T, NN>::tuned; });
+    with_mesh_size(c.N, [&]<int NN>() { t = Lines<T, NN>::tuned; });
     return t;
 }
 
@@ -356,7 +326,7 @@ int tune_col_pass(Ctx &c, int pass)
     for (int v = 0; v < NCOLSHAPES; v++) {
         c.col_shape[pass] = v;
         auto run = [&]() {
-            with_fast_n(N, [&]<int NN>() {
+            with_mesh_size(N, [&]<int NN>() {
                 using F = FastPasses<T, NN>;
                 if (pass == 0) {
                     F::template cols<false>(c, 9, p, -1);
@@ -392,7 +362,7 @@ bool fft_tune_shapes(Ctx &c, int force_y, int force_z)
         c.col_shape[0] = c.col_shape[1] = 0;
         return false;
     }
-    with_fast_n(c.N, [&]<int NN>() { FastPasses<T, NN>::attrs(); });
+    with_mesh_size(c.N, [&]<int NN>() { FastPasses<T, NN>::attrs(); });
     if (force_y < 0 || force_z < 0) {
         // the spectra hold nothing between steps; clear them so the timed transforms see finite data
         cudaMemsetAsync(c.spec, 0, 9 * 2 * sizeof(T) * (size_t)c.nh, c.stream);

@@ -9,6 +9,7 @@
 
 #include "../../include/pm.h"
 #include "pm_once.cuh"
+#include "pm_sizes.cuh"
 
 namespace pm {
 

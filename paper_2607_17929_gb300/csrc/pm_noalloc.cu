@@ -89,15 +89,6 @@ __global__ void k_na_contrast(double *rho, int64_t nc)
     if (i < nc) rho[i] -= 1.0;
 }
 
-bool na_valid_mesh(int n)
-{
-    if (n < 8 || n > NA_MAX_MESH || n % 8) return false;
-    int m = n;
-    while (m % 2 == 0) m /= 2;
-    while (m % 3 == 0) m /= 3;
-    return m == 1;
-}
-
 }  // namespace
 }  // namespace pm
 
@@ -108,7 +99,7 @@ extern "C" pm_status pm_power_spectrum_noalloc(const double *d_pos, int64_t n_pa
     if (!d_pos || !k || !pk || !nmodes || n_part < 1 || n_part >= ((int64_t)1 << 31) || !(omega_m > 0.0) ||
         nbins < 2)
         return PM_ERR_INVALID_ARG;
-    if (!na_valid_mesh(n_mesh) || nbins > NA_MAX_BINS) return PM_ERR_UNSUPPORTED_SIZE;
+    if (!is_mesh_size(n_mesh) || n_mesh > NA_MAX_MESH || nbins > NA_MAX_BINS) return PM_ERR_UNSUPPORTED_SIZE;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= NA_MAX_DEVICES) {
         cudaGetLastError();
