@@ -656,7 +656,7 @@ template <class T, bool FULL, bool DEN> struct DepCol {
         if (lane >= nx) r.prev = r.mid = r.end;   // nothing
         return r;
     }
-    // the row's first 32 records, into part `par` of the stage
+    // the row's records from c0 on, 32 at most, into part `par` of the stage
     __device__ __forceinline__ void fetch_row(int par, const DepRow &r, int c0 = 0)
     {
         const int i = c0 + (threadIdx.x & 31);
@@ -665,7 +665,7 @@ template <class T, bool FULL, bool DEN> struct DepCol {
 #pragma unroll
             for (int q = 0; q < PQ; q++) {
                 const unsigned a = (unsigned)__cvta_generic_to_shared(stage + (par * PQ + q) * DEP_THREADS + threadIdx.x);
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(a), "l"(g + q));
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(a), "l"(g + q) : "memory");
             }
         }
     }
@@ -756,14 +756,14 @@ template <class T, bool FULL, bool DEN> struct DepCol {
                 P = unpack(stage + PAR * PQ * DEP_THREADS + threadIdx.x, DEP_THREADS);
                 if (i >= r.nh) cx = P.cell - base;
             }
-            if (r.total - c0 > 32) {   // the row's next records
-                fetch_row(PAR, r, c0 + 32);
-                asm volatile("cp.async.commit_group;" ::: "memory");
-            }
             T wt[8], q00, q[8], ex;
             charges<T, FULL>(p, P, lo + cx, up + cx, wt, q00, q, ex);
             if (iz >= 0 && w > 0 && i >= r.nh && i < r.total) k0.add(ex);
             __syncwarp();
+            if (r.total - c0 > 32) {   // the row's next records, over those used above
+                fetch_row(PAR, r, c0 + 32);
+                asm volatile("cp.async.commit_group;" ::: "memory");
+            }
 #pragma unroll
             for (int k = 0; k < 8 / VT; k++) rv[32 * k + lane] = pack(wt + VT * k);
             if constexpr (FULL) {
