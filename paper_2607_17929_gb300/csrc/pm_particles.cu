@@ -1044,6 +1044,7 @@ template <class T> struct KdParams {
 constexpr int KROWS = 8, KD_THREADS = 32 * KROWS;
 constexpr int KPX = 32 + 3, KPN = KPX * (KROWS + 3);   // vertices of a plane
 constexpr int KRING = 5;
+constexpr int KUNEVEN = 96;   // FP32: particles of a row from which its tile's warps share their rows
 constexpr int KLD = (KPN + KD_THREADS - 1) / KD_THREADS;   // vertices of a plane per thread
 
 // phi, chi, B_x, B_y of one vertex in one 16-byte (FP32) or two 16-byte (FP64) loads
@@ -1187,12 +1188,14 @@ __device__ __forceinline__ bool carry_cells(double v, int N, double &f, int &car
 }
 __device__ __forceinline__ bool carry_cells(float, int, float &, int &) { return false; }
 
-// FP64: the particles of the rows of cells of a plane.  An FP64 instruction takes the pipe as long for one lane as for
-// 32, so where a row has more than 32 particles, or all rows so few that most lanes would be idle, the warps share all
-// rows' particles in groups of 32 (128^3, own rows and shared ones: z = 1 1.89 -> 1.46 ms, half a particle a cell 1.21 ->
-// 0.72, 0.05 0.98 -> 0.36, a tenth of the mass in cells of 1000 2.39 -> 1.44).  From 192 particles a plane on, 6 of 8
-// full groups, there is nothing to gain.  FP32 kernels keep their own rows: with the table they were slower at one
-// particle a cell (256^3 0.46 -> 0.52 ms), which the rows of more than 32 do not make up for (z = 1 0.70 -> 0.71).
+// The particles of the rows of cells of a plane, for the warps to share in groups of 32 where a row has more than 32, or
+// all rows so few that most lanes would be idle.  FP64, where an instruction takes the pipe as long for one lane as for 32,
+// always keeps this table (128^3, own rows and shared ones: z = 1 1.89 -> 1.46 ms, half a particle a cell 1.21 -> 0.72,
+// 0.05 0.98 -> 0.36, a tenth of the mass in cells of 1000 2.39 -> 1.44; from 192 particles a plane on, 6 of 8 full groups,
+// there is nothing to gain).  FP32 is slower with it at one particle a cell (256^3 0.46 -> 0.52), so only the relativistic
+// kernel takes it, in tiles with a row of more than KUNEVEN (128^3, clumps as above 0.196 -> 0.110, of 300 0.157 -> 0.106,
+// 192^3 at z = 1 0.358 -> 0.349); to look for one costs the other tiles 2% (512^3 3.47 -> 3.55).  In the Newtonian kernel,
+// half as long, both forms together spill and cost 19%.
 struct alignas(16) KickRows {
     int end[KROWS];   // particles of the rows up to this one
     int off[KROWS];   // particle j of all rows' is off[its row] + j
@@ -1237,8 +1240,8 @@ struct alignas(16) KickRows {
 };
 static_assert(KROWS == 8, "find() compares with 7 ends");
 
-// CORR: with the force correction of a Newtonian context
-template <class T, bool NEWT, bool CORR = false>
+// CORR: with the force correction of a Newtonian context.  SHARED: with a table of the rows
+template <class T, bool NEWT, bool CORR, bool SHARED>
 __device__ __forceinline__ void kick_tile(const KdParams<T> &p, const int b)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -1291,16 +1294,16 @@ __device__ __forceinline__ void kick_tile(const KdParams<T> &p, const int b)
         keep(i);
     }
     const int32_t *st = p.start + z0 * (N * N) + y0 * N + x0;
-    __shared__ KickRows rows[FP64 ? 4 : 1];   // FP64 only
+    __shared__ KickRows rows[SHARED ? 4 : 1];
     // this lane's first particle of a plane, fetched a plane ahead
     V nxt[PQ];
     auto fetch = [&](int i) {
 #pragma unroll
         for (int q = 0; q < PQ; q++) nxt[q] = reinterpret_cast<const V *>(p.part + i)[q];
     };
-    int i0 = -1, r0 = w;                  // FP64: that particle and its row
-    int s0 = 0, e0 = 0, s1 = 0, e1 = 0;   // FP32: this warp's row in this plane and the next
-    if constexpr (FP64) {   // the rows of a plane are counted two planes ahead, by a warp after the other
+    int i0 = -1, r0 = w;                  // SHARED: that particle and its row
+    int s0 = 0, e0 = 0, s1 = 0, e1 = 0;   // else this warp's row in this plane and the next
+    if constexpr (SHARED) {   // the rows of a plane are counted two planes ahead, by a warp after the other
         const int32_t *q = st + w * (N * N) + (lane % KROWS) * N;
         if (w < 2 && w < nz) rows[w].set(__ldg(q), __ldg(q + nx));
         __syncthreads();
@@ -1322,10 +1325,10 @@ __device__ __forceinline__ void kick_tile(const KdParams<T> &p, const int b)
     for (int iz = 0; iz < nz; iz++) {
         const int z = z0 + iz;
         if (iz + 1 < nz) load(z + 3);
-        const bool ahead = iz + 2 < nz && (!FP64 || w == iz % KROWS);
+        const bool ahead = iz + 2 < nz && (!SHARED || w == iz % KROWS);
         int s2 = 0, e2 = 0;
         if (ahead) {
-            const int32_t *q = st + (iz + 2) * (N * N) + (FP64 ? lane % KROWS : w) * N;
+            const int32_t *q = st + (iz + 2) * (N * N) + (SHARED ? lane % KROWS : w) * N;
             s2 = __ldg(q);
             e2 = __ldg(q + nx);
         }
@@ -1333,7 +1336,7 @@ __device__ __forceinline__ void kick_tile(const KdParams<T> &p, const int b)
 #pragma unroll
         for (int q = 0; q < PQ; q++) rec[q] = nxt[q];
         int i = i0, r = r0;
-        if constexpr (FP64) {
+        if constexpr (SHARED) {
             i0 = -1;
             if (iz + 1 < nz) rows[(iz + 1) % 4].first(w, (w + z + 1) % KROWS, i0, r0);
             if (i0 >= 0) fetch(i0);
@@ -1422,7 +1425,7 @@ __device__ __forceinline__ void kick_tile(const KdParams<T> &p, const int b)
             p.part[i] = P;
             atomicAdd(&p.count[P.cell], 1);
         };
-        if constexpr (FP64) {
+        if constexpr (SHARED) {
             const KickRows &now = rows[iz % 4];
             for (unsigned c = 32 * ((unsigned)(w + z) % KROWS);;) {
                 if (i >= 0) move(i, r);
@@ -1441,7 +1444,7 @@ __device__ __forceinline__ void kick_tile(const KdParams<T> &p, const int b)
         // plane z + 3 into the slot of plane z - 2, last read before the barrier of the plane before
         if (iz + 1 < nz) keep(sc + 4 >= KRING ? sc + 4 - KRING : sc + 4);
         __syncthreads();
-        if constexpr (!FP64) {
+        if constexpr (!SHARED) {
             s0 = s1;
             e0 = e1;
             s1 = s2;
@@ -1451,13 +1454,35 @@ __device__ __forceinline__ void kick_tile(const KdParams<T> &p, const int b)
     }
 }
 
+// Whether a row of the tile has more than KUNEVEN particles, for the whole CTA.
+template <class T> __device__ __forceinline__ bool kick_uneven(const KdParams<T> &p, const int b)
+{
+    const int N = p.N, x0 = (b % p.ntx) * p.nrow, y0 = ((b / p.ntx) % (N / KROWS)) * KROWS, z0 = b / (p.ntx * (N / KROWS)) * p.tz;
+    const int nx = min(p.nrow, N - x0), nz = min(p.tz, N - z0);
+    int most = 0;
+    for (int r = threadIdx.x; r < KROWS * nz; r += KD_THREADS) {
+        const int32_t *q = p.start + ((z0 + r / KROWS) * N + y0 + r % KROWS) * N + x0;
+        most = max(most, __ldg(q + nx) - __ldg(q));
+    }
+    return __syncthreads_or(most > KUNEVEN);
+}
+
+template <class T, bool NEWT, bool CORR = false>
+__device__ __forceinline__ void kick_cells(const KdParams<T> &p, const int b)
+{
+    if constexpr (sizeof(T) == 8) kick_tile<T, NEWT, CORR, true>(p, b);
+    else if constexpr (NEWT) kick_tile<T, NEWT, CORR, false>(p, b);
+    else if (kick_uneven(p, b)) kick_tile<T, NEWT, CORR, true>(p, b);
+    else kick_tile<T, NEWT, CORR, false>(p, b);
+}
+
 // CTAs an SM holds: the relativistic FP32 kernel needs 80 registers, the Newtonian one 64, FP64 128
 template <class T, bool NEWT> constexpr int kd_ctas() { return sizeof(T) == 4 ? (NEWT ? 4 : 3) : 2; }
 
 template <class T, bool NEWT>
 __global__ void __launch_bounds__(KD_THREADS, kd_ctas<T, NEWT>()) k_kick_drift(const __grid_constant__ KdParams<T> p)
 {
-    kick_tile<T, NEWT>(p, blockIdx.x);
+    kick_cells<T, NEWT>(p, blockIdx.x);
 }
 
 // The Newtonian kick with a force correction: one pass over the particles instead of k_corr_kick's before it
@@ -1465,7 +1490,7 @@ __global__ void __launch_bounds__(KD_THREADS, kd_ctas<T, NEWT>()) k_kick_drift(c
 template <class T>
 __global__ void __launch_bounds__(KD_THREADS, sizeof(T) == 4 ? 3 : 2) k_kick_corrected(const __grid_constant__ KdParams<T> p)
 {
-    kick_tile<T, true, true>(p, blockIdx.x);
+    kick_cells<T, true, true>(p, blockIdx.x);
 }
 
 template <class T> struct KdBatch {
@@ -1480,7 +1505,7 @@ __global__ void __launch_bounds__(KD_THREADS, kd_ctas<T, NEWT>()) k_kick_batch(c
 {
     int i = 0;
     while (i + 1 < q.nbox && (int)blockIdx.x >= q.first[i + 1]) i++;
-    kick_tile<T, NEWT>(q.box[i], (int)blockIdx.x - q.first[i]);
+    kick_cells<T, NEWT>(q.box[i], (int)blockIdx.x - q.first[i]);
 }
 
 // ---------------------------------------------------------------------------

@@ -84,3 +84,35 @@ def test_mass_deposit_of_a_dense_load(pm):  # noqa: F811
     stages full cells one after another."""
     t = [stage_ms(make(pm, pm.PM_MIXED, pm.PM_NEWTONIAN, c), "project") / c for c in (1, 16)]
     assert t[1] < 1.1 * t[0], t
+
+
+def test_mixed_kick_of_clumps(pm):  # noqa: F811
+    """A tenth of the mass in cells of 1000: 1.3 times the even load; 2 where each warp takes its own row."""
+    t = [stage_ms(make(pm, pm.PM_MIXED, 0, 1.0, c), "kick_drift") for c in (0, 1000)]
+    assert t[1] < 1.6 * t[0], t
+
+
+def test_mixed_clumps_move_as_in_fp64(pm):  # noqa: F811
+    """Rows of far more than 96 particles beside ordinary ones, tiles with and without: every particle is moved once.
+    Momenta of the mixed step to its bound, positions to 1e-5 of a cell (a drift far below a cell)."""
+    import numpy as np
+    from mixed_bounds import MIXED_BOUND
+    from test_parity_gpu import rel
+    rng = np.random.default_rng(17)
+    n = 48
+    cells = np.array([[0, 0, 0], [47, 47, 47], [23, 7, 8], [24, 8, 7], [10, 40, 16]])
+    pos = np.concatenate([c + rng.integers(0, 1 << 24, (m, 3)) / 2.0 ** 24
+                          for c, m in zip(cells, (400, 97, 96, 1000, 33))] +
+                         [rng.integers(0, n, (n ** 3, 3)) + rng.integers(0, 1 << 24, (n ** 3, 3)) / 2.0 ** 24]) / n
+    mom = (1e-3 * rng.standard_normal(pos.shape)).astype(np.float32).astype(np.float64)
+    got = []
+    for prec in (pm.PM_FP64, pm.PM_MIXED):
+        g = pm.PM(n, len(pos), 10.0 * n, 0.31, 20.0, 0.0, 100, prec)
+        g.set_particles(pos, mom)
+        for _ in range(2):
+            g.step()
+        got.append(g.particles())
+        g.close()
+    (x0, u0), (x1, u1) = got
+    assert rel(u1, u0) < MIXED_BOUND["u"] and np.abs((x1 - x0 + 0.5) % 1.0 - 0.5).max() * n < 1e-5
+    assert np.abs(x1 - pos).max() > 0 and (u1 != mom).any(1).all()
