@@ -45,9 +45,10 @@ template <class T, int N, bool ZP = false, int V = 0> struct Lines {
     static constexpr int col = col1 * TLC > 1024 ? 1024 / TLC : col1;
     // Row pairs per block of the x passes: 256 threads, 128 for sizes with a factor of three.  Those hold
     // 24 points a thread, few warps fit an SM, and every exchange stops the whole block: smaller blocks
-    // leave others to run meanwhile (r2c / c2r, us, FP32 192^3: 354 / 206 with 256 threads, 316 / 185
-    // with 128; 288^3: 1277 / 758, 1196 / 721; 72^3: 32 / 38, 29 / 28; FP64 192^3: 3875 / 2112, 3631 /
-    // 1927; 64 threads gain no more).  With 8 points a thread it makes no difference (256^3: 458 / 279, 461 / 274).
+    // leave others to run meanwhile (one r2c launch of 9 fields / one c2r launch of 5, us, with 256 and with 128
+    // threads: FP32 192^3 170 / 97 and 152 / 88; 288^3 614 / 343 and 568 / 330; 72^3 16.7 / 18.6 and 16.5 / 14.5;
+    // FP64 192^3 1836 / 959 and 1720 / 878; 64 threads gain no more).  With 8 points a thread they gain nothing
+    // (256^3 220 / 131 and 223 / 128, 512^3 1759 / 1002 and 1816 / 1016).
     static constexpr int row_threads = N % 3 == 0 && TL <= 128 ? 128 : 256;
     static constexpr int row = TL >= 256 ? 1 : row_threads / TL;
     // resident blocks per SM the register allocation must allow

@@ -15,8 +15,9 @@ namespace pm {
 
 // ---------------------------------------------------------------------------
 // Precision traits.  FP64: f64 everywhere.  Mixed: f32 offsets, momenta,
-// fields and FFTs; per-cell deposit sums in compensated f32 (float-float,
-// about 48 significant bits) and the k = 0 mode in f64.
+// fields and FFTs; the deposit's T^00 sums in compensated f32 (float-float
+// with TwoSum, about 48 significant bits for sums of some thousand terms) and
+// the k = 0 mode in f64.
 // ---------------------------------------------------------------------------
 template <class T> struct Cplx;
 template <> struct Cplx<double> { using type = double2; };

@@ -3,13 +3,13 @@
 //
 // Projection (Sec. 2.1 "particle-mesh projection", Eqs. matterstress):
 // particles are kept sorted by cell.  A CTA owns a column of mesh vertices and
-// marches along z, one cell plane at a time: a thread owns one cell of the
-// plane, adds the charges of its particles to the cell's 8 corners in
-// registers, and the corner sums of neighbouring cells meet in registers (z),
-// through a shuffle (x) and through shared memory (y).  No global atomics, and
-// every mesh value is written once.  The same kernel assembles the
-// configuration-space sources of the field equations from phi_{n-1},
-// chi_{n-1}, phi_{n-2}.
+// marches along z, one plane of cells at a time.  A warp takes an x-row of
+// cells: a lane forms the charges of one of its particles, then sums, for one
+// vertex, over the particles of the two cells beside it; the sums of
+// neighbouring planes meet in registers and those of neighbouring rows through
+// shared memory.  No global atomics, and every mesh value is written once.
+// The same kernel assembles the configuration-space sources of the field
+// equations from phi_{n-1}, chi_{n-1}, phi_{n-2}.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -60,11 +60,10 @@ template <> struct Acc<float> {
 };
 
 // 1 / sqrt(x) and a / b: the hardware approximations (a few ulp) in the mixed form, whose
-// FP32 rounding already sets the error; IEEE operations in FP64
+// FP32 rounding already sets the error; CUDA's rsqrt (1 ulp) in FP64
 __device__ __forceinline__ float rsqrt_t(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double rsqrt_t(double x) { return rsqrt(x); }
 __device__ __forceinline__ float div_t(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ double div_t(double a, double b) { return a / b; }
 
 template <class T> __device__ __forceinline__ T mulr(T a, T b);
 template <> __device__ __forceinline__ float mulr<float>(float a, float b) { return __fmul_rn(a, b); }
@@ -270,11 +269,13 @@ template <class I> __global__ void __launch_bounds__(MTHREADS, 4) k_mass(const _
 //  - shared memory carries the y + 1 sums to the next row's warp, which then holds whole vertices.
 // What bounds it: instruction issue (FP32) and the FP64 pipe (FP64).  A particle's charges are formed once per
 // CTA that needs them (about 1.2 times: (nrow + 1)/nrow, (ncol + 1)/ncol and (tz + 1)/tz), its record is read
-// by two vertex lanes, and a vertex costs 36 products per particle of two cells.  Against 8^3 vertex tiles that
+// by two vertex lanes, and a vertex costs 36 products per particle of two cells, in packed pairs in FP32, or, where a
+// cell is full, 3 per lane (crowd_sums).  Against 8^3 vertex tiles that
 // stage the charges of 9^3 cells and let each vertex gather from 8 cells (a record read 8 times, potentials, ranges
-// and a scan set up per tile), at 512^3 mixed 6.9 -> 4.0 ms early (sums of one plane in registers, 40 of them, so
-// 20 warps an SM), at 256^3 FP64 15.3 -> 8.0, late (192^3, z = 1, cells of up to 55 particles) 0.59 -> 0.56.  A cell per lane with its 8 corners in registers was faster early (3.4 ms) but ran as
-// long as its row's fullest cell (late 0.78 ms).
+// and a scan set up per tile), at 512^3 mixed 6.9 -> 3.9 ms early (sums of one plane in registers, 40 of them, so
+// 20 warps an SM), at 256^3 FP64 15.3 -> 8.1, late (192^3, z = 1, cells of up to 55 particles) 0.59 -> 0.58; at 4 and 16
+// particles a cell (128^3) FP32 0.45 -> 0.49 and 1.66 -> 1.95, FP64 7.9 -> 8.2 and 33.8 -> 20.0.  A cell per lane with its
+// 8 corners in registers was faster early (3.4 ms) but ran as long as its row's fullest cell (late 0.78 ms).
 // ---------------------------------------------------------------------------
 constexpr int DROWS = 10;                 // rows of cells of a tile along y, one warp each
 constexpr int DTY = DROWS - 1;            // and of vertices, at most
@@ -978,7 +979,7 @@ __global__ void __launch_bounds__(DEP_THREADS, dep_ctas<T, FULL>()) k_project(co
 
 // The CIC density contrast of the P(k) diagnostic in FP32 contexts: the columns above with the weights and the sums
 // in two words.  In place of FP64 weights and atomics on the FP64 pipe: 256^3 at z = 3 0.98 (with clearing and the
-// final pass) -> 0.55 ms.  FP64 contexts take k_density_acc.
+// final pass) -> 0.48 ms.  FP64 contexts take k_density_acc.
 __global__ void __launch_bounds__(DEP_THREADS, 2) k_contrast(const __grid_constant__ DepParams<float> p)
 {
     deposit_tile<float, false, true>(p, blockIdx.x);
@@ -1038,8 +1039,8 @@ template <class T> struct KdParams {
 // What bounds it: the shared-memory pipe (a particle reads 32 vertices of 20 bytes, 5 of its 8 wavefronts) and, in
 // FP64, the FP64 pipe.  Against 8^3 tiles of 11^3 vertices, one search and three integer divisions per particle, and
 // the gradients of five fields kept in 20 registers (512^3 mixed 5.15 ms, 256^3 FP64 14.0, 288^3 Newtonian 0.52):
-// 3.5 ms, 8.8, 0.29.  Rows that hold more than 32 particles make their CTA's other warps wait (192^3 at z = 1:
-// 0.33 -> 0.33).  Two planes between barriers, records staged in shared memory instead of registers, four CTAs of 64
+// 3.55 ms, 8.8, 0.30.  Rows that hold more than 32 particles make their CTA's other warps wait where they are not shared
+// (192^3 at z = 1: 0.33 -> 0.35).  Two planes between barriers, records staged in shared memory instead of registers, four CTAs of 64
 // registers an SM, two of 128: 0.58, 0.48, 0.61, 0.52 ms against 0.46 at 256^3 (the first two take L1 from the loads).
 constexpr int KROWS = 8, KD_THREADS = 32 * KROWS;
 constexpr int KPX = 32 + 3, KPN = KPX * (KROWS + 3);   // vertices of a plane
@@ -2104,7 +2105,9 @@ void launch_project_batch(Ctx *const *cs, const StepScalars *ss, int n, bool ful
 }
 
 // Tiles of the kick: rows of up to 32 cells, as long along z as makes the number of waves times (tz + 2) smallest
-// (the fields of three more planes are loaded than cells are visited).
+// (the fields of three more planes are loaded than cells are visited).  A wave is counted with the relativistic kernel's
+// CTAs (three an SM in FP32) for the Newtonian one, too, which holds four: with four, 128^3 and 192^3 gain 1-4%, 144^3 and
+// 288^3 lose 3-4% (0.336 -> 0.346 ms).
 template <class T> KdParams<T> kd_params(const Ctx &c, const StepScalars &s)
 {
     KdParams<T> p{};
